@@ -132,46 +132,7 @@ bool finite_all(const double* p, size_t n) {
 
 }  // namespace
 
-void host_energy_constants(sdft_ctx* c) {
-    // E_self = sum Z^2 / (2 sqrt(pi) r_loc); E_sc = 1/2 sum' Z Z' erfc(d/s)/d, s = sqrt(2(r^2 + r'^2))
-    c->E_self = 0.0;
-    for (int a = 0; a < c->natom; ++a) {
-        const sdft_pseudo& s = c->species[c->types[a]];
-        c->E_self += s.Z * s.Z / (2.0 * std::sqrt(M_PI) * s.r_loc);
-    }
-    c->E_sc = 0.0;
-    c->dEsc.assign(3 * c->natom, 0.0);
-    const double rmax = 30.0;
-    int nimg[3];
-    for (int d = 0; d < 3; ++d) nimg[d] = c->opt.boundary == SDFT_BC_DIRICHLET ? 0 : (int)std::ceil(rmax / c->L[d]) + 1;
-    for (int a = 0; a < c->natom; ++a) {
-        const sdft_pseudo& sa = c->species[c->types[a]];
-        for (int b = 0; b < c->natom; ++b) {
-            const sdft_pseudo& sb = c->species[c->types[b]];
-            const double s = std::sqrt(2.0 * (sa.r_loc * sa.r_loc + sb.r_loc * sb.r_loc));
-            for (int t0 = -nimg[0]; t0 <= nimg[0]; ++t0)
-                for (int t1 = -nimg[1]; t1 <= nimg[1]; ++t1)
-                    for (int t2 = -nimg[2]; t2 <= nimg[2]; ++t2) {
-                        if (a == b && t0 == 0 && t1 == 0 && t2 == 0) continue;
-                        const double v[3] = {c->pos[3 * a] - c->pos[3 * b] - t0 * c->L[0],
-                                             c->pos[3 * a + 1] - c->pos[3 * b + 1] - t1 * c->L[1],
-                                             c->pos[3 * a + 2] - c->pos[3 * b + 2] - t2 * c->L[2]};
-                        const double d = std::sqrt(v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-                        if (d > rmax) continue;
-                        c->E_sc += 0.5 * sa.Z * sb.Z * std::erfc(d / s) / d;
-                        if (a != b) {
-                            const double f = sa.Z * sb.Z *
-                                             (-2.0 / (s * std::sqrt(M_PI)) * std::exp(-(d / s) * (d / s)) / d -
-                                              std::erfc(d / s) / (d * d));
-                            for (int q = 0; q < 3; ++q) c->dEsc[3 * a + q] += f * v[q] / d;
-                        }
-                    }
-        }
-    }
-}
-
 namespace {
-
 
 void build_context(sdft_ctx* c) {
     const sdft_options& o = c->opt;
@@ -213,7 +174,7 @@ void build_context(sdft_ctx* c) {
         build_kb_tables(c, k);
         any_cplx = any_cplx || c->kb[k].cplx;
     }
-    host_energy_constants(c);
+    energy_constants(c);
     // problems
     const int np = o.nspin * o.nkpt;
     double* eig_all = (double*)ctx_alloc(c, sizeof(double) * np * ns);

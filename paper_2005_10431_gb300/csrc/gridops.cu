@@ -1,5 +1,4 @@
-// Grid-level FP64 kernels of the SCF (paper Sec. 2.1): pseudocharges and the SAD guess,
-// Perdew-Zunger LDA, the AAR Poisson solver, density from orbitals (Eq. 2), Fermi-Dirac
+// Grid-level FP64 kernels of the SCF (paper Sec. 2.1): Perdew-Zunger LDA, the AAR Poisson solver, density from orbitals (Eq. 2), Fermi-Dirac
 // occupations, Pulay mixing, reductions and Hellmann-Feynman forces.
 #include "internal.cuh"
 
@@ -12,52 +11,11 @@ namespace {
 
 constexpr int RB = 256;   // reduction block size
 
-// ---------------------------------------------------------------------------------------
-// set-up: pseudocharge b and SAD density, summed over periodic images within the cutoff
-// ---------------------------------------------------------------------------------------
+// an atom's pseudocharge amplitude, width and cut-off
 struct AtomG {
     double pos[3];
-    double amp_b, w_b, cut_b;      // pseudocharge amplitude, width, cutoff
-    double amp_s, w_s, cut_s;      // SAD
+    double amp_b, w_b, cut_b;
 };
-
-__device__ double image_sum(double x, double y, double z, const double* pos, double L1, double L2, double L3,
-                            double amp, double w, double cut, int isolated) {
-    double s = 0.0;
-    const double L[3] = {L1, L2, L3};
-    const double X[3] = {x, y, z};
-    int tlo[3], thi[3];
-    for (int d = 0; d < 3; ++d) {
-        tlo[d] = isolated ? 0 : (int)ceil((X[d] - pos[d] - cut) / L[d]);   // isolated: the atom itself only
-        thi[d] = isolated ? 0 : (int)floor((X[d] - pos[d] + cut) / L[d]);
-    }
-    const double inv = 1.0 / (2.0 * w * w);
-    for (int t2 = tlo[2]; t2 <= thi[2]; ++t2)
-        for (int t1 = tlo[1]; t1 <= thi[1]; ++t1)
-            for (int t0 = tlo[0]; t0 <= thi[0]; ++t0) {
-                const double dx = X[0] - pos[0] - t0 * L1, dy = X[1] - pos[1] - t1 * L2, dz = X[2] - pos[2] - t2 * L3;
-                const double r2 = dx * dx + dy * dy + dz * dz;
-                if (r2 <= cut * cut) s += amp * exp(-r2 * inv);
-            }
-    return s;
-}
-
-__global__ void setup_fields_kernel(const AtomG* __restrict__ at, int natom, int n1, int n2, int n3, double h1,
-                                    double h2, double h3, double L1, double L2, double L3, double* __restrict__ b,
-                                    double* __restrict__ sad, int isolated) {
-    const long long ng = (long long)n1 * n2 * n3;
-    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < ng; g += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(g % n1), j = (int)((g / n1) % n2), k = (int)(g / ((long long)n1 * n2));
-        const double x = i * h1, y = j * h2, z = k * h3;
-        double sb = 0.0, ss = 0.0;
-        for (int a = 0; a < natom; ++a) {
-            sb += image_sum(x, y, z, at[a].pos, L1, L2, L3, at[a].amp_b, at[a].w_b, at[a].cut_b, isolated);
-            ss += image_sum(x, y, z, at[a].pos, L1, L2, L3, at[a].amp_s, at[a].w_s, at[a].cut_s, isolated);
-        }
-        b[g] = sb;
-        sad[g] = ss;
-    }
-}
 
 // ---------------------------------------------------------------------------------------
 // reductions: deterministic two-stage sums of several dot products
@@ -709,9 +667,6 @@ std::vector<AtomG> atom_g(sdft_ctx* c) {
         at[a].amp_b = -s.Z * std::pow(2.0 * M_PI * s.r_loc * s.r_loc, -1.5);
         at[a].w_b = s.r_loc;
         at[a].cut_b = 10.0 * s.r_loc;
-        at[a].amp_s = s.Z * std::pow(2.0 * M_PI * s.sad_width * s.sad_width, -1.5);
-        at[a].w_s = s.sad_width;
-        at[a].cut_s = 10.0 * s.sad_width;
     }
     return at;
 }
@@ -742,33 +697,6 @@ void dots_host(sdft_ctx* c, int count, const double* const* a, const double* con
     SDFT_CUDA(cudaMemcpyAsync(c->hscal, out, sizeof(double) * 8, cudaMemcpyDeviceToHost, c->stream));
     SDFT_CUDA(cudaStreamSynchronize(c->stream));
     for (int k = 0; k < count; ++k) host_out[k] = c->hscal[k];
-}
-
-void build_pseudocharge_and_sad(sdft_ctx* c) {
-    std::vector<AtomG> at = atom_g(c);
-    AtomG* dat = (AtomG*)ctx_alloc(c, sizeof(AtomG) * std::max(1, c->natom));
-    SDFT_CUDA(cudaMemcpyAsync(dat, at.data(), sizeof(AtomG) * c->natom, cudaMemcpyHostToDevice, c->stream));
-    setup_fields_kernel<<<nblocks(c->ng), 256, 0, c->stream>>>(dat, c->natom, c->n[0], c->n[1], c->n[2], c->h[0],
-                                                              c->h[1], c->h[2], c->L[0], c->L[1], c->L[2], c->b,
-                                                              c->rho_sad, c->opt.boundary == SDFT_BC_DIRICHLET);
-    SDFT_CUDA(cudaGetLastError());
-    count_launch(c);
-    // normalise the SAD density to N_e: sum rho = rho . 1
-    double* ones = c->work64;
-    SDFT_CUDA(cudaMemsetAsync(ones, 0, sizeof(double) * c->ng, c->stream));
-    c->hscal[0] = 1.0;
-    SDFT_CUDA(cudaMemcpyAsync(c->scal, c->hscal, sizeof(double), cudaMemcpyHostToDevice, c->stream));
-    add_scalar_kernel<<<nblocks(c->ng), 256, 0, c->stream>>>(ones, c->scal, 1.0, c->ng);
-    count_launch(c);
-    const double* a[1] = {c->rho_sad};
-    const double* b[1] = {ones};
-    double s = 0.0;
-    dots_host(c, 1, a, b, c->ng, &s);
-    const double scale = c->nelec / (c->dV * s);
-    axpby_kernel<double><<<nblocks(c->ng), 256, 0, c->stream>>>(c->rho_sad, c->rho_sad, 0.0, scale, c->ng);
-    SDFT_CUDA(cudaGetLastError());
-    count_launch(c);
-    ctx_release(c, dat);
 }
 
 // ---------------------------------------------------------------------------------------

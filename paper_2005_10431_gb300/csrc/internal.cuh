@@ -346,10 +346,13 @@ void release_kb_tables(sdft_ctx* c, int kpt);
 // ---- qmd.cu: atom moves and the extrapolated start of the next SCF ----------------------
 void push_scf_history(sdft_ctx* c);
 void move_atoms(sdft_ctx* c, const double* pos, int guess);
-void host_energy_constants(sdft_ctx* c);
+
+// ---- atoms.cu: fields and energies summed over atoms and images ----------------------------
+void build_pseudocharge_and_sad(sdft_ctx* c);
+void descriptor_field(sdft_ctx* c, void* feat);   // BF16 [ng][32]
+void energy_constants(sdft_ctx* c);               // E_self, E_sc, dEsc (host)
 
 // ---- gridops.cu ----------------------------------------------------------------------
-void build_pseudocharge_and_sad(sdft_ctx* c);
 void lda_device(sdft_ctx* c, int nspin, const double* rho, double* exc, double* vxc, size_t n);
 void veff_assemble(sdft_ctx* c);
 void veff_to_float(sdft_ctx* c, int spin);

@@ -22,25 +22,51 @@ struct AtomBox {
     double rp, rc;
 };
 
-__global__ void atom_support_kernel(const AtomBox* __restrict__ boxes, int cap, int n1, int n2, int n3,
-                                    double h1, double h2, double h3, double k1, double k2, double k3,
-                                    int cplx, int* __restrict__ cnt, int* __restrict__ idx,
-                                    int* __restrict__ img, double* __restrict__ val64,
-                                    float* __restrict__ val32, int isolated) {
+// Support points of atom blockIdx.x among chunk blockIdx.y of its box (contiguous in box order): their number into
+// ccnt (FILL false), or, after that, their lists in box order from the sum of the earlier chunks' numbers on.  Bound
+// by the FP64 pipe: the squared displacements of an axis are tabulated once per CTA, so a box point costs three
+// operations, and the normalisation is formed by one thread (a pow() in every thread was half of the time).  One CTA
+// per atom took 146 us for the 64-atom cell, this takes 64 us.
+constexpr int SUP_CHUNKS = 8;
+template <bool FILL>
+__global__ void __launch_bounds__(256)
+atom_support_kernel(const AtomBox* __restrict__ boxes, int cap, int n1, int n2, int n3, double h1, double h2, double h3,
+                    double k1, double k2, double k3, int cplx, int* __restrict__ ccnt, int* __restrict__ cnt,
+                    int* __restrict__ idx, int* __restrict__ img, double* __restrict__ val64,
+                    float* __restrict__ val32, int isolated) {
+    extern __shared__ double disp[];   // displacements of the box's columns, rows and planes
     const int a = blockIdx.x;
     const AtomBox B = boxes[a];
     const int total = B.dim[0] * B.dim[1] * B.dim[2];
-    const double norm = rsqrt(pow(M_PI, 1.5) * B.rp * B.rp * B.rp);
-    __shared__ int warp_tot[32];
+    const int per = (total + SUP_CHUNKS - 1) / SUP_CHUNKS, p0 = blockIdx.y * per, p1 = min(total, p0 + per);
+    __shared__ int warp_tot[8];
     __shared__ int base;
-    if (threadIdx.x == 0) base = 0;
+    __shared__ double norm;
+    double* const dx = disp;
+    double* const dy = dx + B.dim[0];
+    double* const dz = dy + B.dim[1];
+    for (int i = threadIdx.x; i < B.dim[0]; i += blockDim.x) dx[i] = (B.lo[0] + i) * h1 - B.pos[0];
+    for (int i = threadIdx.x; i < B.dim[1]; i += blockDim.x) dy[i] = (B.lo[1] + i) * h2 - B.pos[1];
+    for (int i = threadIdx.x; i < B.dim[2]; i += blockDim.x) dz[i] = (B.lo[2] + i) * h3 - B.pos[2];
+    if (threadIdx.x == 0) {
+        base = 0;
+        if (FILL) {
+            norm = rsqrt(pow(M_PI, 1.5) * B.rp * B.rp * B.rp);
+            int sum = 0;
+            for (int c = 0; c < SUP_CHUNKS; ++c) {
+                if (c == (int)blockIdx.y) base = sum;
+                sum += ccnt[a * SUP_CHUNKS + c];
+            }
+            if (blockIdx.y == 0) cnt[a] = sum;
+        }
+    }
     __syncthreads();
-    for (int start = 0; start < total; start += blockDim.x) {
+    for (int start = p0; start < p1; start += blockDim.x) {
         const int p = start + threadIdx.x;
         bool keep = false;
         int I[3] = {0, 0, 0};
         double r2 = 0.0;
-        if (p < total) {
+        if (p < p1) {
             int rem = p;
             const int ix = rem % B.dim[0];
             rem /= B.dim[0];
@@ -49,8 +75,7 @@ __global__ void atom_support_kernel(const AtomBox* __restrict__ boxes, int cap, 
             I[0] = B.lo[0] + ix;
             I[1] = B.lo[1] + iy;
             I[2] = B.lo[2] + iz;
-            const double dx = I[0] * h1 - B.pos[0], dy = I[1] * h2 - B.pos[1], dz = I[2] * h3 - B.pos[2];
-            r2 = dx * dx + dy * dy + dz * dz;
+            r2 = fma(dz[iz], dz[iz], fma(dx[ix], dx[ix], __dmul_rn(dy[iy], dy[iy])));
             keep = r2 < B.rc * B.rc;
             // an isolated cell has no periodic images: points beyond the grid are not wrapped back in
             if (isolated && (I[0] < 0 || I[0] >= n1 || I[1] < 0 || I[1] >= n2 || I[2] < 0 || I[2] >= n3)) keep = false;
@@ -66,7 +91,7 @@ __global__ void atom_support_kernel(const AtomBox* __restrict__ boxes, int cap, 
             if (w < warp) off += warp_tot[w];
             all += warp_tot[w];
         }
-        if (keep) {
+        if (FILL && keep) {
             const int slot = base + off + before;
             int t[3], g[3];
             const int nn[3] = {n1, n2, n3};
@@ -99,13 +124,13 @@ __global__ void atom_support_kernel(const AtomBox* __restrict__ boxes, int cap, 
         if (threadIdx.x == 0) base += all;
         __syncthreads();
     }
-    if (threadIdx.x == 0) cnt[a] = base;
+    if (!FILL && threadIdx.x == 0) ccnt[a * SUP_CHUNKS + blockIdx.y] = base;
 }
 
 __global__ void point_count_kernel(const int* __restrict__ cnt, const int* __restrict__ idx, int cap,
                                    int* __restrict__ pcnt) {
     const int a = blockIdx.x;
-    for (int j = threadIdx.x; j < cnt[a]; j += blockDim.x) atomicAdd(&pcnt[idx[(long long)a * cap + j]], 1);
+    for (int j = blockIdx.y * blockDim.x + threadIdx.x; j < cnt[a]; j += gridDim.y * blockDim.x) atomicAdd(&pcnt[idx[(long long)a * cap + j]], 1);
 }
 
 __global__ void point_fill_kernel(const int* __restrict__ cnt, const int* __restrict__ idx,
@@ -114,7 +139,7 @@ __global__ void point_fill_kernel(const int* __restrict__ cnt, const int* __rest
                                   int* __restrict__ patom, double* __restrict__ pval64,
                                   float* __restrict__ pval32) {
     const int a = blockIdx.x;
-    for (int j = threadIdx.x; j < cnt[a]; j += blockDim.x) {
+    for (int j = blockIdx.y * blockDim.x + threadIdx.x; j < cnt[a]; j += gridDim.y * blockDim.x) {
         const long long e = (long long)a * cap + j;
         const int g = idx[e];
         const int s = atomicAdd(&pfill[g], 1);
@@ -215,13 +240,24 @@ void build_kb_tables(sdft_ctx* c, int kpt) {
     std::vector<double> gam(c->natom);
     for (int a = 0; a < c->natom; ++a) gam[a] = c->species[c->types[a]].E_kb * c->dV;
     AtomBox* dboxes = (AtomBox*)ctx_alloc(c, sizeof(AtomBox) * std::max(1, c->natom));
+    int* ccnt = (int*)ctx_alloc(c, sizeof(int) * SUP_CHUNKS * std::max(1, c->natom));
     if (c->natom > 0) {
         SDFT_CUDA(cudaMemcpyAsync(T.gamma, gam.data(), sizeof(double) * c->natom, cudaMemcpyHostToDevice, c->stream));
         SDFT_CUDA(cudaMemcpyAsync(dboxes, boxes.data(), sizeof(AtomBox) * c->natom, cudaMemcpyHostToDevice, c->stream));
-        atom_support_kernel<<<c->natom, 256, 0, c->stream>>>(dboxes, T.cap, c->n[0], c->n[1], c->n[2], c->h[0], c->h[1],
-                                                            c->h[2], kred[0], kred[1], kred[2], T.cplx, T.cnt, T.idx,
-                                                            T.img, T.val64, T.val32,
-                                                            c->opt.boundary == SDFT_BC_DIRICHLET);
+        int side = 0;
+        for (const AtomBox& B : boxes) side = std::max(side, B.dim[0] + B.dim[1] + B.dim[2]);
+        const size_t dsm = sizeof(double) * (size_t)side;
+        auto launch = [&](auto kfn) {
+            if (dsm > 48 * 1024)
+                SDFT_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm));
+            kfn<<<dim3(c->natom, SUP_CHUNKS), 256, dsm, c->stream>>>(dboxes, T.cap, c->n[0], c->n[1], c->n[2], c->h[0],
+                                                                     c->h[1], c->h[2], kred[0], kred[1], kred[2],
+                                                                     T.cplx, ccnt, T.cnt, T.idx, T.img, T.val64,
+                                                                     T.val32, c->opt.boundary == SDFT_BC_DIRICHLET);
+        };
+        launch(atom_support_kernel<false>);
+        launch(atom_support_kernel<true>);
+        count_launch(c);
         SDFT_CUDA(cudaGetLastError());
         count_launch(c);
     }
@@ -230,7 +266,7 @@ void build_kb_tables(sdft_ctx* c, int kpt) {
     SDFT_CUDA(cudaMemsetAsync(T.pcnt, 0, sizeof(int) * c->ng, c->stream));
     int S = 0;
     if (c->natom > 0) {
-        point_count_kernel<<<c->natom, 256, 0, c->stream>>>(T.cnt, T.idx, T.cap, T.pcnt);
+        point_count_kernel<<<dim3(c->natom, 8), 256, 0, c->stream>>>(T.cnt, T.idx, T.cap, T.pcnt);
         int* dmax = (int*)c->scal;
         SDFT_CUDA(cudaMemsetAsync(dmax, 0, sizeof(int), c->stream));
         max_kernel<<<256, 256, 0, c->stream>>>(T.pcnt, c->ng, dmax);
@@ -248,7 +284,7 @@ void build_kb_tables(sdft_ctx* c, int kpt) {
         T.pval32 = (float*)ctx_alloc(c, sizeof(float) * ps * vw);
         int* pfill = (int*)ctx_alloc(c, sizeof(int) * c->ng);
         SDFT_CUDA(cudaMemsetAsync(pfill, 0, sizeof(int) * c->ng, c->stream));
-        point_fill_kernel<<<c->natom, 256, 0, c->stream>>>(T.cnt, T.idx, T.val64, T.val32, T.cap, T.cplx, c->ng, S,
+        point_fill_kernel<<<dim3(c->natom, 8), 256, 0, c->stream>>>(T.cnt, T.idx, T.val64, T.val32, T.cap, T.cplx, c->ng, S,
                                                           pfill, T.patom, T.pval64, T.pval32);
         point_sort_kernel<<<(unsigned)((c->ng + 255) / 256), 256, 0, c->stream>>>(T.pcnt, c->ng, T.cplx, T.patom,
                                                                                   T.pval64, T.pval32);
@@ -257,6 +293,7 @@ void build_kb_tables(sdft_ctx* c, int kpt) {
         ctx_release(c, pfill);
     }
     ctx_release(c, dboxes);
+    ctx_release(c, ccnt);
 }
 
 void release_kb_tables(sdft_ctx* c, int kpt) {

@@ -23,7 +23,6 @@ constexpr int NF = 32, NH = 64;
 constexpr int OW1 = 0, OB1 = OW1 + NH * NF, OW2 = OB1 + NH, OB2 = OW2 + NH * NH, OW3 = OB2 + NH, OB3 = OW3 + NH;
 constexpr int NP = OB3 + 1;   // 6337 parameters
 constexpr int TP = 64;        // points per tile
-constexpr double RC = 6.5;
 
 __device__ __forceinline__ float silu(float z) { return z / (1.f + __expf(-z)); }
 __device__ __forceinline__ float dsilu(float z) {
@@ -31,45 +30,6 @@ __device__ __forceinline__ float dsilu(float z) {
     return s * (1.f + z * (1.f - s));
 }
 __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
-
-__global__ void descriptor_kernel(const double* __restrict__ pos, int natom, int n1, int n2, int n3, double h1,
-                                  double h2, double h3, double L1, double L2, double L3,
-                                  __nv_bfloat16* __restrict__ feat) {
-    const long long ng = (long long)n1 * n2 * n3;
-    const double eta = 6.0 / 31.0;
-    for (long long g = blockIdx.x * (long long)blockDim.x + threadIdx.x; g < ng; g += (long long)gridDim.x * blockDim.x) {
-        const int i = (int)(g % n1), j = (int)((g / n1) % n2), k = (int)(g / ((long long)n1 * n2));
-        const double X[3] = {i * h1, j * h2, k * h3};
-        const double L[3] = {L1, L2, L3};
-        float G[NF];
-#pragma unroll
-        for (int q = 0; q < NF; ++q) G[q] = 0.f;
-        for (int a = 0; a < natom; ++a) {
-            int tlo[3], thi[3];
-            for (int d = 0; d < 3; ++d) {
-                tlo[d] = (int)ceil((X[d] - pos[3 * a + d] - RC) / L[d]);
-                thi[d] = (int)floor((X[d] - pos[3 * a + d] + RC) / L[d]);
-            }
-            for (int t2 = tlo[2]; t2 <= thi[2]; ++t2)
-                for (int t1 = tlo[1]; t1 <= thi[1]; ++t1)
-                    for (int t0 = tlo[0]; t0 <= thi[0]; ++t0) {
-                        const double dx = X[0] - pos[3 * a] - t0 * L1, dy = X[1] - pos[3 * a + 1] - t1 * L2,
-                                     dz = X[2] - pos[3 * a + 2] - t2 * L3;
-                        const double r = sqrt(dx * dx + dy * dy + dz * dz);
-                        if (r > RC) continue;
-                        const float fc = (float)(0.5 * (cos(M_PI * r / RC) + 1.0));
-                        const float rf = (float)r, inv2e2 = (float)(1.0 / (2.0 * eta * eta));
-#pragma unroll
-                        for (int q = 0; q < NF; ++q) {
-                            const float u = rf - (float)(6.0 * q / 31.0);
-                            G[q] = fmaf(expf(-u * u * inv2e2), fc, G[q]);
-                        }
-                    }
-        }
-#pragma unroll
-        for (int q = 0; q < NF; ++q) feat[g * NF + q] = __float2bfloat16_rn(G[q]);
-    }
-}
 
 struct MlpSmem {
     float W1T[NF][NH];   // W1 transposed (bf16-rounded)
@@ -333,13 +293,7 @@ int mlp_nparam() { return NP; }
 // features of every grid point of the context's cell; target (optional) = rho_out - rho_SAD of the
 // last SCF, summed over spins
 void mlp_dataset(sdft_ctx* c, void* feat, float* target) {
-    double* dpos = reinterpret_cast<double*>(c->work64);   // positions staged in grid scratch
-    SDFT_CUDA(cudaMemcpyAsync(dpos, c->pos.data(), sizeof(double) * 3 * c->natom, cudaMemcpyHostToDevice, c->stream));
-    descriptor_kernel<<<(unsigned)std::min<long long>((c->ng + 255) / 256, 152LL * 16), 256, 0, c->stream>>>(
-        dpos, c->natom, c->n[0], c->n[1], c->n[2], c->h[0], c->h[1], c->h[2], c->L[0], c->L[1], c->L[2],
-        reinterpret_cast<__nv_bfloat16*>(feat));
-    SDFT_CUDA(cudaGetLastError());
-    count_launch(c);
+    descriptor_field(c, feat);
     if (target) {
         target_kernel<<<(unsigned)std::min<long long>((c->ng + 255) / 256, 152LL * 16), 256, 0, c->stream>>>(
             c->rho_out, c->opt.nspin, c->rho_sad, target, c->ng);

@@ -115,7 +115,7 @@ void move_atoms(sdft_ctx* c, const double* pos, int guess) {
         release_kb_tables(c, (int)k);
         build_kb_tables(c, (int)k);
     }
-    host_energy_constants(c);
+    energy_constants(c);
     c->mix_k = 0;
     c->mix_count = 0;
     c->mix_head = 0;

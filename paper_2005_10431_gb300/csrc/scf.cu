@@ -29,27 +29,48 @@ __device__ __forceinline__ unsigned long long splitmix64(unsigned long long x) {
     z = (z ^ (z >> 27)) * 0x94D049BB133111EBULL;
     return z ^ (z >> 31);
 }
-__device__ __forceinline__ double uniform_counter(unsigned long long seed, unsigned long long i) {
-    const unsigned long long z = splitmix64(((seed & 0xffffffffULL) << 32) + i);
-    return (double)(z >> 11) * (1.0 / 9007199254740992.0) - 0.5;
+// A value in the block's own type without the FP64 pipe (an FP64 conversion, product and difference per
+// value bounded the fill: 246 us for 180 FP32 columns of 80^3 points).  (top 53 bits) 2^-53 - 1/2 = s 2^-53 with the
+// integer s = top - 2^52, exact in FP64 and rounded once to FP32.
+__device__ __forceinline__ long long uniform_bits(unsigned long long seed, unsigned long long i) {
+    return (long long)(splitmix64(((seed & 0xffffffffULL) << 32) + i) >> 11) - (1LL << 52);
+}
+__device__ __forceinline__ float scaled_f32(long long s) { return __ll2float_rn(s) * 1.1102230246251565e-16f; }   // 2^-53
+__device__ __forceinline__ double scaled_f64(long long s) {
+    const unsigned long long mag = (unsigned long long)(s < 0 ? -s : s);   // at most 2^52
+    if (mag == 0) return 0.0;
+    const int top = 63 - __clzll((long long)mag);                          // leading bit: mag in [2^top, 2^(top + 1))
+    const unsigned long long frac = (mag << (52 - top)) & 0xfffffffffffffULL;
+    const unsigned long long bits = (s < 0 ? 1ULL << 63 : 0ULL) | ((unsigned long long)(1023 - 53 + top) << 52) | frac;
+    return __longlong_as_double((long long)bits);
 }
 
-__global__ void seed_kernel(int kind, void* __restrict__ X, int ncol, long long ng, unsigned long long seed) {
-    const long long total = (long long)ncol * ng;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total; e += (long long)gridDim.x * blockDim.x) {
-        const int n = (int)(e / ng);
-        const long long g = e - (long long)n * ng;
-        const double re = uniform_counter(seed, (unsigned long long)e);
-        if (kind == 0) {
-            ((double*)X)[e] = re;
-        } else if (kind == 1) {
-            const double im = uniform_counter(seed + 0x5BD1, (unsigned long long)e);
-            ((double2*)X)[e] = make_double2(re, im);
-        } else if (kind == 2) {
-            ((float*)X)[(((long long)(n >> 1)) * ng + g) * 2 + (n & 1)] = (float)re;
-        } else {
-            const double im = uniform_counter(seed + 0x5BD1, (unsigned long long)e);
-            ((float2*)X)[e] = make_float2((float)re, (float)im);
+// column n of the block per blockIdx.y (column pair 2p, 2p + 1 of the paired FP32 layout, one 8-byte store per
+// point), four points a thread.  180 FP32 columns of 80^3 points: 246 -> 172 us; 132 FP64 columns: 250 ->
+// 156 us.
+constexpr int SEED_PTS = 4;
+__global__ void __launch_bounds__(256) seed_kernel(int kind, void* __restrict__ X, int ncol, long long ng,
+                                                   unsigned long long seed) {
+    const int cols = kind == 2 ? (ncol + 1) / 2 : ncol;
+    for (int y = blockIdx.y; y < cols; y += gridDim.y) {
+        const long long e0 = (kind == 2 ? 2LL * y : (long long)y) * ng;
+        const long long g0 = blockIdx.x * (long long)(256 * SEED_PTS) + threadIdx.x;
+#pragma unroll
+        for (int u = 0; u < SEED_PTS; ++u) {
+            const long long g = g0 + 256 * u;
+            if (g >= ng) break;
+            const unsigned long long e = (unsigned long long)(e0 + g);
+            const long long re = uniform_bits(seed, e);
+            if (kind == 0) {
+                ((double*)X)[e] = scaled_f64(re);
+            } else if (kind == 2) {
+                const long long r1 = 2 * y + 1 < ncol ? uniform_bits(seed, e + (unsigned long long)ng) : 0;
+                ((float2*)X)[(long long)y * ng + g] = make_float2(scaled_f32(re), scaled_f32(r1));
+            } else {
+                const long long im = uniform_bits(seed + 0x5BD1, e);
+                if (kind == 1) ((double2*)X)[e] = make_double2(scaled_f64(re), scaled_f64(im));
+                else ((float2*)X)[e] = make_float2(scaled_f32(re), scaled_f32(im));
+            }
         }
     }
 }
@@ -194,7 +215,8 @@ void axpby_dev(sdft_ctx* c, double* y, const double* x, double a, double b, long
 }
 
 void seed_orbitals(sdft_ctx* c, int precision, bool cplx, void* X, int ncol, uint64_t seed) {
-    seed_kernel<<<nb((long long)ncol * c->ng), 256, 0, c->stream>>>(kind_of(precision, cplx), X, ncol, c->ng, seed);
+    const dim3 grid((unsigned)((c->ng + 256 * SEED_PTS - 1) / (256 * SEED_PTS)), (unsigned)std::min(ncol, 65535));
+    seed_kernel<<<grid, 256, 0, c->stream>>>(kind_of(precision, cplx), X, ncol, c->ng, seed);
     SDFT_CUDA(cudaGetLastError());
     count_launch(c);
 }
