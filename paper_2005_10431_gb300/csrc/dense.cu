@@ -154,43 +154,83 @@ gram_kernel(const void* __restrict__ Y, const void* __restrict__ HY, int ncol, l
         }
 }
 
-// sum the split-K partials (upper triangle), mirror to a full Hermitian matrix
-__global__ void gram_reduce_kernel(const double* __restrict__ part, int nsplit, int ncol, int cplx,
-                                   double* __restrict__ M, double* __restrict__ Hs) {
+// Sum the split-K partials (upper triangle) and mirror to a full Hermitian matrix.  A 20-state matrix has 210
+// sums of up to 432 terms: one thread per element walking through them was one memory latency per term (310 us
+// complex, 77 us for 8 states).  LANES threads now share an element's terms of one matrix, eight loads in flight
+// each: 20 complex columns 310 -> 14 us, 8 FP64 columns 77 -> 28 us.  FP64 kinds keep one thread per sum (LANES = 1, 16 loads in flight) and with it the order of
+// the additions, so FP64 results are the same bit for bit as before; the FP32 kinds' partials carry FP32 rounding.
+// grid.y: matrix (M, Hs); W = 2 for complex.
+template <int LANES, int W>
+__global__ void __launch_bounds__(256)
+gram_reduce_kernel(const double* __restrict__ part, int nsplit, int ncol, double* __restrict__ M,
+                   double* __restrict__ Hs) {
     const long long nn = (long long)ncol * ncol;
-    const int w = cplx ? 2 : 1;
-    for (long long o = blockIdx.x * (long long)blockDim.x + threadIdx.x; o < nn; o += (long long)gridDim.x * blockDim.x) {
+    double* __restrict__ out = blockIdx.y == 0 ? M : Hs;
+    const double* __restrict__ p0 = part + blockIdx.y * nn * W;
+    const long long t0 = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    const int sub = (int)(t0 % LANES);
+    for (long long o = t0 / LANES; o < nn; o += (long long)gridDim.x * (blockDim.x / LANES)) {
         const int i = (int)(o % ncol), j = (int)(o / ncol);
-        if (j < i) continue;
-        double m[2] = {0, 0}, h[2] = {0, 0};
-        for (int s = 0; s < nsplit; ++s) {
-            const double* pm = part + (long long)s * 2 * nn * w;
-            const double* ph = pm + nn * w;
-            for (int q = 0; q < w; ++q) {
-                m[q] += pm[w * o + q];
-                h[q] += ph[w * o + q];
+        double v[W];
+#pragma unroll
+        for (int q = 0; q < W; ++q) v[q] = 0.0;
+        if (j >= i) {
+            // U terms are added while the next U are on their way; terms past the end are zeros, not loads
+            constexpr int U = LANES == 1 ? 16 : 8;
+            double t[2][U][W];
+            auto load = [&](int s, double (*d)[W]) {
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int q = 0; q < W; ++q)
+                        d[u][q] = s + u * LANES < nsplit ? p0[(long long)(s + u * LANES) * 2 * nn * W + W * o + q] : 0.0;
+            };
+            load(sub, t[0]);
+            for (int s = sub; s < nsplit; s += 2 * U * LANES) {
+                load(s + U * LANES, t[1]);
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int q = 0; q < W; ++q) v[q] += t[0][u][q];
+                load(s + 2 * U * LANES, t[0]);
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int q = 0; q < W; ++q) v[q] += t[1][u][q];
             }
         }
+        if (LANES > 1) {   // an element's lanes are neighbours in one warp and leave the loop together
+#pragma unroll
+            for (int off = LANES / 2; off > 0; off >>= 1)
+#pragma unroll
+                for (int q = 0; q < W; ++q)
+                    v[q] += __shfl_down_sync(__activemask(), v[q], off, LANES);
+        }
+        if (sub != 0 || j < i) continue;
         const long long ot = (long long)j + (long long)i * ncol;
-        if (cplx) {
-            M[2 * o] = m[0];
-            M[2 * o + 1] = m[1];
-            M[2 * ot] = m[0];
-            M[2 * ot + 1] = -m[1];
-            Hs[2 * o] = h[0];
-            Hs[2 * o + 1] = h[1];
-            Hs[2 * ot] = h[0];
-            Hs[2 * ot + 1] = -h[1];
-            if (i == j) {
-                M[2 * o + 1] = 0.0;
-                Hs[2 * o + 1] = 0.0;
-            }
+        if (W == 2) {
+            out[2 * o] = v[0];
+            out[2 * ot] = v[0];
+            out[2 * o + 1] = i == j ? 0.0 : v[W - 1];
+            if (i != j) out[2 * ot + 1] = -v[W - 1];
         } else {
-            M[o] = m[0];
-            M[ot] = m[0];
-            Hs[o] = h[0];
-            Hs[ot] = h[0];
+            out[o] = v[0];
+            out[ot] = v[0];
         }
+    }
+}
+
+void launch_gram_reduce(int kind, const double* part, int nsplit, int ncol, double* M, double* Hs, cudaStream_t st) {
+    const long long nn = (long long)ncol * ncol;
+    auto launch = [&](auto kfn, int lanes) {
+        const dim3 grid((unsigned)std::min<long long>((nn * lanes + 255) / 256, 152LL * 16), 2);
+        kfn<<<grid, 256, 0, st>>>(part, nsplit, ncol, M, Hs);
+    };
+    switch (kind) {
+        case 0: launch(gram_reduce_kernel<1, 1>, 1); break;
+        case 1: launch(gram_reduce_kernel<1, 2>, 1); break;
+        case 2: launch(gram_reduce_kernel<8, 1>, 8); break;
+        default: launch(gram_reduce_kernel<8, 2>, 8); break;
     }
 }
 
@@ -366,7 +406,7 @@ void subspace_gram_noalloc(int precision, bool cplx, const void* Y, const void* 
         case 2: gram_kernel<2><<<grid, 256, 0, stream>>>(Y, HY, ncol, ng, chunk, part); break;
         default: gram_kernel<3><<<grid, 256, 0, stream>>>(Y, HY, ncol, ng, chunk, part); break;
     }
-    gram_reduce_kernel<<<nb(nn), 256, 0, stream>>>(part, (int)nsplit, ncol, cplx, M, Hs);
+    launch_gram_reduce(kind, part, (int)nsplit, ncol, M, Hs, stream);
     SDFT_CUDA(cudaGetLastError());
 }
 
@@ -398,7 +438,7 @@ void subspace_gram(sdft_ctx* c, int precision, bool cplx, const void* Y, const v
         case 2: gram_kernel<2><<<grid, 256, 0, c->stream>>>(Y, HY, ncol, c->ng, chunk, c->part); break;
         default: gram_kernel<3><<<grid, 256, 0, c->stream>>>(Y, HY, ncol, c->ng, chunk, c->part); break;
     }
-    gram_reduce_kernel<<<nb(nn), 256, 0, c->stream>>>(c->part, (int)nsplit, ncol, cplx, M, Hs);
+    launch_gram_reduce(kind, c->part, (int)nsplit, ncol, M, Hs, c->stream);
     SDFT_CUDA(cudaGetLastError());
     count_launch(c, 2);
 }
