@@ -238,61 +238,46 @@ size_t eig32_smem(int n) {
 }
 
 // C = op(A) B for n x n column-major FP64 matrices, op(A) = A or A^T; blockIdx.z picks one of
-// two products.  32 x 32 tile per CTA, 2 x 2 outputs per thread.
+// two products.  Bound by the SMs' two FP64 multiply-adds per clock, so the tile is small: at n = 180 tiles of 32
+// gave 36 CTAs a product (62 us for two products or one), tiles of 16 give 144, one output per thread (21 to 27 us
+// for a launch).  The additions over k are in order either way.
 struct Prod2 {
     const double* A[2];
     const double* B[2];
     double* C[2];
 };
 
+constexpr int G64_T = 16;
 template <bool TA>
-__global__ void __launch_bounds__(256) gemm64_kernel(Prod2 g, int n, const int* __restrict__ status) {
-    constexpr int T = 32, KT = 16;
+__global__ void __launch_bounds__(G64_T * G64_T) gemm64_kernel(Prod2 g, int n, const int* __restrict__ status) {
+    constexpr int T = G64_T;
     if (*status & ST_CHOLESKY) return;
-    __shared__ double As[KT][T + 1];   // As[k][i] = op(A)(i0 + i, k0 + k)
-    __shared__ double Bs[KT][T + 1];   // Bs[k][j] = B(k0 + k, j0 + j)
+    __shared__ double As[T][T + 1];   // As[k][i] = op(A)(i0 + i, k0 + k)
+    __shared__ double Bs[T][T + 1];   // Bs[j][k] = B(k0 + k, j0 + j)
     const double* __restrict__ A = g.A[blockIdx.z];
     const double* __restrict__ B = g.B[blockIdx.z];
     double* __restrict__ C = g.C[blockIdx.z];
     const int i0 = blockIdx.x * T, j0 = blockIdx.y * T;
-    const int tx = threadIdx.x % 16, ty = threadIdx.x / 16;
-    double acc[2][2] = {{0.0, 0.0}, {0.0, 0.0}};
-    for (int k0 = 0; k0 < n; k0 += KT) {
-        for (int e = threadIdx.x; e < KT * T; e += 256) {
-            int i, k;
-            if (TA) {
-                k = e % KT;
-                i = e / KT;
-            } else {
-                i = e % T;
-                k = e / T;
-            }
-            const int gi = i0 + i, gk = k0 + k;
-            double v = 0.0;
-            if (gi < n && gk < n) v = TA ? A[gk + (long long)gi * n] : A[gi + (long long)gk * n];
-            As[k][i] = v;
-            const int kb = e % KT, jb = e / KT;
-            const int gj = j0 + jb, gkb = k0 + kb;
-            Bs[kb][jb] = (gj < n && gkb < n) ? B[gkb + (long long)gj * n] : 0.0;
-        }
+    const int tx = threadIdx.x % T, ty = threadIdx.x / T;
+    // the next tiles are on their way while this one is multiplied
+    auto load = [&](int k0, double& a, double& b) {
+        const int gi = i0 + (TA ? ty : tx), gk = k0 + (TA ? tx : ty);
+        a = gi < n && gk < n ? (TA ? A[gk + (long long)gi * n] : A[gi + (long long)gk * n]) : 0.0;
+        b = j0 + ty < n && k0 + tx < n ? B[k0 + tx + (long long)(j0 + ty) * n] : 0.0;
+    };
+    double a, b, acc = 0.0;
+    load(0, a, b);
+    for (int k0 = 0; k0 < n; k0 += T) {
+        As[TA ? tx : ty][TA ? ty : tx] = a;
+        Bs[ty][tx] = b;
         __syncthreads();
+        if (k0 + T < n) load(k0 + T, a, b);
 #pragma unroll
-        for (int k = 0; k < KT; ++k) {
-            const double a0 = As[k][tx], a1 = As[k][tx + 16], b0 = Bs[k][ty], b1 = Bs[k][ty + 16];
-            acc[0][0] = fma(a0, b0, acc[0][0]);
-            acc[1][0] = fma(a1, b0, acc[1][0]);
-            acc[0][1] = fma(a0, b1, acc[0][1]);
-            acc[1][1] = fma(a1, b1, acc[1][1]);
-        }
+        for (int k = 0; k < T; ++k) acc = fma(As[k][tx], Bs[ty][k], acc);
         __syncthreads();
     }
-#pragma unroll
-    for (int a = 0; a < 2; ++a)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            const int i = i0 + tx + 16 * a, j = j0 + ty + 16 * b;
-            if (i < n && j < n) C[i + (long long)j * n] = acc[a][b];
-        }
+    const int i = i0 + tx, j = j0 + ty;
+    if (i < n && j < n) C[i + (long long)j * n] = acc;
 }
 
 __device__ __forceinline__ void atomic_max_nonneg(unsigned long long* p, double v) {
@@ -305,171 +290,188 @@ __device__ double block_max(double v, unsigned long long* slot) {
     return v;
 }
 
-// steps 2 (mode 0) and 3 (mode 1): T from G = Q^T M Q and S = Q^T Hs Q; mode 1 also writes the
-// eigenvalues (ascending) and checks the final residuals.  ws: 2 * RE_KMAX * n doubles.
-__global__ void __launch_bounds__(1024, 1)
-refine_step_kernel(const double* __restrict__ G, const double* __restrict__ S, double* __restrict__ Tm,
-                   double* __restrict__ eig, double* __restrict__ ws, int n, int step, int mode,
-                   int* __restrict__ status, double* __restrict__ diag) {
-    __shared__ double lam[RE2_MAX_N];
-    __shared__ int ord[RE2_MAX_N], rnk[RE2_MAX_N], first[RE2_MAX_N], cstart[RE2_MAX_N], csize[RE2_MAX_N];
-    __shared__ unsigned long long s_eta, s_scale, s_inter, s_orth;
-    __shared__ int s_bad;
+// Steps 2 (mode 0) and 3 (mode 1): T from G = Q^T M Q and S = Q^T Hs Q; mode 1 also writes the eigenvalues
+// (ascending) and checks the final residuals.  The n^2 passes (maxima, T) run one column per CTA over the whole GPU;
+// only the ordering and the cluster bounds, O(n) data, are one CTA's (all of it in one CTA was 168 us a step at
+// n = 180, bound by that SM's FP64 pipe; at most 26 us now).
+struct RefineState {
+    double lam[RE2_MAX_N];
+    int ord[RE2_MAX_N], cluster[RE2_MAX_N];     // index of the r-th eigenvalue; cluster (its first rank) of index i
+    int first[RE2_MAX_N], csize[RE2_MAX_N];     // rank r starts a cluster, of this size
+    double omega;                               // cluster threshold, set by the first step
+    unsigned long long mx[4];                   // bit patterns of eta, scale, inter, orth
+    int bad;
+};
+
+// column j = blockIdx.x: lam_j, the largest off-diagonal residual and |lam|
+__global__ void __launch_bounds__(128) refine_max_kernel(const double* __restrict__ G, const double* __restrict__ S, int n,
+                                                         const int* __restrict__ status, RefineState* __restrict__ R) {
     if (*status & ST_CHOLESKY) return;
-    const int tid = threadIdx.x, NT = blockDim.x;
-    const int warp = tid >> 5, lane = tid & 31, nwarp = NT >> 5;
-    const long long nn = (long long)n * n;
-    if (tid == 0) {
-        s_eta = s_scale = s_inter = s_orth = 0ull;
-        s_bad = 0;
+    const int j = blockIdx.x;
+    const double* __restrict__ Gj = G + (long long)j * n;
+    const double* __restrict__ Sj = S + (long long)j * n;
+    double l = Sj[j] / Gj[j];
+    if (!isfinite(l)) {
+        if (threadIdx.x == 0) R->bad = 1;
+        l = 0.0;
     }
-    __syncthreads();
-    for (int i = tid; i < n; i += NT) {
-        double l = S[i + (long long)i * n] / G[i + (long long)i * n];
-        if (!isfinite(l)) {
-            s_bad = 1;
-            l = 0.0;
-        }
-        lam[i] = l;
-    }
-    __syncthreads();
-    double eta = 0.0, sc = 0.0;
-    for (int j = warp; j < n; j += nwarp)
-        for (int i = lane; i < n; i += 32) {
-            const long long e = i + (long long)j * n;
-            if (i != j) eta = fmax(eta, fabs(S[e] - lam[j] * G[e]));
-            else sc = fmax(sc, fabs(lam[i]));
-        }
+    double eta = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x)
+        if (i != j) eta = fmax(eta, fabs(Sj[i] - l * Gj[i]));
     if (!isfinite(eta)) {
-        s_bad = 1;
+        R->bad = 1;
         eta = 0.0;
     }
-    block_max(eta, &s_eta);
-    block_max(sc, &s_scale);
+    block_max(eta, &R->mx[0]);
+    if (threadIdx.x == 0) {
+        R->lam[j] = l;
+        atomic_max_nonneg(&R->mx[1], fabs(l));
+    }
+}
+
+// order of the lam, cluster threshold and clusters
+__global__ void __launch_bounds__(1024, 1) refine_order_kernel(int n, int step, int* __restrict__ status,
+                                                               RefineState* __restrict__ R) {
+    __shared__ double lam[RE2_MAX_N];
+    __shared__ long long key[RE2_MAX_N];   // lam as integers of the same order: ranking stays off the FP64 pipe
+    __shared__ int ord[RE2_MAX_N], first[RE2_MAX_N];
+    if (*status & ST_CHOLESKY) return;
+    const int tid = threadIdx.x, NT = blockDim.x;
+    for (int i = tid; i < n; i += NT) {
+        lam[i] = R->lam[i];
+        const long long b = __double_as_longlong(lam[i] + 0.0);
+        key[i] = b < 0 ? (long long)0x8000000000000000ULL - b : b;
+    }
+    __syncthreads();
     for (int i = tid; i < n; i += NT) {
         int r = 0;
-        for (int j = 0; j < n; ++j) r += (lam[j] < lam[i]) || (lam[j] == lam[i] && j < i);
-        rnk[i] = r;
+        for (int j = 0; j < n; ++j) r += (key[j] < key[i]) || (key[j] == key[i] && j < i);
         ord[r] = i;
     }
     __syncthreads();
-    const double scale = __longlong_as_double((long long)s_scale);
-    // cluster threshold: set by the first step, kept by the later ones (diag[8])
-    const double omega = step == 0 ? fmax(100.0 * __longlong_as_double((long long)s_eta), 1e-14 * fmax(scale, 1e-300))
-                                   : diag[8];
+    const double scale = __longlong_as_double((long long)R->mx[1]);
+    // cluster threshold: set by the first step, kept by the later ones
+    const double omega = step == 0 ? fmax(100.0 * __longlong_as_double((long long)R->mx[0]), 1e-14 * fmax(scale, 1e-300))
+                                   : R->omega;
     for (int r = tid; r < n; r += NT) first[r] = r == 0 || lam[ord[r]] - lam[ord[r - 1]] > omega;
     __syncthreads();
     for (int r = tid; r < n; r += NT) {
         int s = r;
         while (!first[s]) --s;
-        cstart[r] = s;
+        R->cluster[ord[r]] = s;
+        R->ord[r] = ord[r];
+        R->first[r] = first[r];
         if (first[r]) {
             int k = 1;
             while (r + k < n && !first[r + k]) ++k;
-            csize[r] = k;
+            R->csize[r] = k;
         }
     }
-    __syncthreads();
-    // off-cluster residual and orthonormality defect of the current Q
-    double inter = 0.0, orth = 0.0;
-    for (int j = warp; j < n; j += nwarp)
-        for (int i = lane; i < n; i += 32) {
-            const long long e = i + (long long)j * n;
-            if (i != j && cstart[rnk[i]] != cstart[rnk[j]]) inter = fmax(inter, fabs(S[e] - lam[j] * G[e]));
-            orth = fmax(orth, fabs(G[e] - (i == j ? 1.0 : 0.0)));
-        }
-    block_max(inter, &s_inter);
-    block_max(orth, &s_orth);
-    if (mode == 0) {
-        for (int j = warp; j < n; j += nwarp)
-            for (int i = lane; i < n; i += 32) {
-            const long long e = i + (long long)j * n;
-            double t;
-            if (i == j) t = 1.0 + 0.5 * (1.0 - G[e]);
-            else if (cstart[rnk[i]] == cstart[rnk[j]]) t = -0.5 * G[e];
-            else t = (S[e] - lam[j] * G[e]) / (lam[j] - lam[i]);
-            Tm[e] = t;
-            }
-    } else {
-        for (long long e = tid; e < nn; e += NT) Tm[e] = 0.0;
-        __syncthreads();
-        for (int r0 = tid; r0 < n; r0 += NT) {
-            if (!first[r0]) continue;
-            const int k = csize[r0];
-            if (k == 1) {
-                const int i = ord[r0];
-                Tm[i + (long long)r0 * n] = 1.0 / sqrt(G[i + (long long)i * n]);
-                eig[r0] = lam[i];
-                continue;
-            }
-            if (k > RE_KMAX) {
-                atomicOr(status, ST_CLUSTER);
-                continue;
-            }
-            double* Bm = ws + (size_t)2 * RE_KMAX * r0;   // k x k, then W (k x k)
-            double* W = Bm + k * k;
-            for (int b = 0; b < k; ++b)
-                for (int a = 0; a < k; ++a) {
-                    const int i = ord[r0 + a], j = ord[r0 + b];
-                    const double gij = sqrt(G[i + (long long)i * n] * G[j + (long long)j * n]);
-                    Bm[a + b * k] = 0.5 * (S[i + (long long)j * n] + S[j + (long long)i * n]) / gij;
-                    W[a + b * k] = a == b ? 1.0 : 0.0;
-                }
-            for (int sweep = 0; sweep < RE_CL_SWEEPS; ++sweep) {
-                int rot = 0;
-                for (int p = 0; p < k - 1; ++p)
-                    for (int q = p + 1; q < k; ++q) {
-                        const double apq = Bm[p + q * k], app = Bm[p + p * k], aqq = Bm[q + q * k];
-                        if (!(fabs(apq) > 1e-16 * (fabs(app) + fabs(aqq)) && fabs(apq) > 1e-300)) continue;
-                        double c, s;
-                        jacobi_cs(app, aqq, apq, c, s);
-                        ++rot;
-                        for (int x = 0; x < k; ++x) {
-                            const double u = Bm[x + p * k], v = Bm[x + q * k];
-                            Bm[x + p * k] = c * u - s * v;
-                            Bm[x + q * k] = s * u + c * v;
-                            const double wu = W[x + p * k], wv = W[x + q * k];
-                            W[x + p * k] = c * wu - s * wv;
-                            W[x + q * k] = s * wu + c * wv;
-                        }
-                        for (int x = 0; x < k; ++x) {
-                            const double u = Bm[p + x * k], v = Bm[q + x * k];
-                            Bm[p + x * k] = c * u - s * v;
-                            Bm[q + x * k] = s * u + c * v;
-                        }
-                    }
-                if (rot == 0) break;
-            }
-            for (int b = 0; b < k; ++b) {
-                const double mu = Bm[b + b * k];
-                int rb = 0;
-                for (int a = 0; a < k; ++a) {
-                    const double ma = Bm[a + a * k];
-                    rb += (ma < mu) || (ma == mu && a < b);
-                }
-                eig[r0 + rb] = mu;
-                for (int a = 0; a < k; ++a) {
-                    const int i = ord[r0 + a];
-                    Tm[i + (long long)(r0 + rb) * n] = W[a + b * k] / sqrt(G[i + (long long)i * n]);
-                }
-            }
-        }
-    }
-    __syncthreads();
     if (tid == 0) {
-        const double e = __longlong_as_double((long long)s_eta), in = __longlong_as_double((long long)s_inter),
-                     o = __longlong_as_double((long long)s_orth);
-        diag[4 * mode + 0] = e;
-        diag[4 * mode + 1] = in;
-        diag[4 * mode + 2] = o;
-        diag[4 * mode + 3] = scale;
-        if (step == 0) diag[8] = omega;
-        int st = s_bad ? ST_NONFINITE : 0;
-        if (mode == 1) {
-            if (!(in <= 1e-10 * fmax(scale, 1.0))) st |= ST_RESIDUAL;
-            if (!(o <= 1e-10)) st |= ST_ORTHO;
+        if (step == 0) R->omega = omega;
+        if (R->bad) atomicOr(status, ST_NONFINITE);
+    }
+}
+
+// column j = blockIdx.x: off-cluster residual and orthonormality defect of the current Q, and T (mode 1: zeroed)
+__global__ void __launch_bounds__(128) refine_fill_kernel(const double* __restrict__ G, const double* __restrict__ S,
+                                                          double* __restrict__ Tm, int n, int mode,
+                                                          const int* __restrict__ status, RefineState* __restrict__ R) {
+    if (*status & ST_CHOLESKY) return;
+    const int j = blockIdx.x, cj = R->cluster[j];
+    const double lj = R->lam[j];
+    double inter = 0.0, orth = 0.0;
+    for (int i = threadIdx.x; i < n; i += blockDim.x) {
+        const long long e = i + (long long)j * n;
+        const double g = G[e], res = S[e] - lj * g;
+        const bool same = R->cluster[i] == cj;
+        if (i != j && !same) inter = fmax(inter, fabs(res));
+        orth = fmax(orth, fabs(g - (i == j ? 1.0 : 0.0)));
+        double t = 0.0;
+        if (mode == 0) {
+            if (i == j) t = 1.0 + 0.5 * (1.0 - g);
+            else if (same) t = -0.5 * g;
+            else t = res / (lj - R->lam[i]);
         }
+        Tm[e] = t;
+    }
+    block_max(inter, &R->mx[2]);
+    block_max(orth, &R->mx[3]);
+}
+
+// mode 1: the Rayleigh-Ritz inside the cluster that starts at rank r0, one thread each; the residual checks
+__global__ void __launch_bounds__(32)
+refine_cluster_kernel(const double* __restrict__ G, const double* __restrict__ S, double* __restrict__ Tm,
+                      double* __restrict__ eig, double* __restrict__ ws, int n, int* __restrict__ status,
+                      const RefineState* __restrict__ R) {
+    if (*status & ST_CHOLESKY) return;
+    const int* __restrict__ ord = R->ord;
+    const int r0 = blockIdx.x * blockDim.x + threadIdx.x;
+    if (r0 == 0) {
+        const double scale = __longlong_as_double((long long)R->mx[1]);
+        int st = 0;
+        if (!(__longlong_as_double((long long)R->mx[2]) <= 1e-10 * fmax(scale, 1.0))) st |= ST_RESIDUAL;
+        if (!(__longlong_as_double((long long)R->mx[3]) <= 1e-10)) st |= ST_ORTHO;
         if (st) atomicOr(status, st);
+    }
+    if (r0 >= n || !R->first[r0]) return;
+    const int k = R->csize[r0];
+    if (k == 1) {
+        const int i = ord[r0];
+        Tm[i + (long long)r0 * n] = 1.0 / sqrt(G[i + (long long)i * n]);
+        eig[r0] = R->lam[i];
+        return;
+    }
+    if (k > RE_KMAX) {
+        atomicOr(status, ST_CLUSTER);
+        return;
+    }
+    double* Bm = ws + (size_t)2 * RE_KMAX * r0;   // k x k, then W (k x k)
+    double* W = Bm + k * k;
+    for (int b = 0; b < k; ++b)
+        for (int a = 0; a < k; ++a) {
+            const int i = ord[r0 + a], j = ord[r0 + b];
+            const double gij = sqrt(G[i + (long long)i * n] * G[j + (long long)j * n]);
+            Bm[a + b * k] = 0.5 * (S[i + (long long)j * n] + S[j + (long long)i * n]) / gij;
+            W[a + b * k] = a == b ? 1.0 : 0.0;
+        }
+    for (int sweep = 0; sweep < RE_CL_SWEEPS; ++sweep) {
+        int rot = 0;
+        for (int p = 0; p < k - 1; ++p)
+            for (int q = p + 1; q < k; ++q) {
+                const double apq = Bm[p + q * k], app = Bm[p + p * k], aqq = Bm[q + q * k];
+                if (!(fabs(apq) > 1e-16 * (fabs(app) + fabs(aqq)) && fabs(apq) > 1e-300)) continue;
+                double c, s;
+                jacobi_cs(app, aqq, apq, c, s);
+                ++rot;
+                for (int x = 0; x < k; ++x) {
+                    const double u = Bm[x + p * k], v = Bm[x + q * k];
+                    Bm[x + p * k] = c * u - s * v;
+                    Bm[x + q * k] = s * u + c * v;
+                    const double wu = W[x + p * k], wv = W[x + q * k];
+                    W[x + p * k] = c * wu - s * wv;
+                    W[x + q * k] = s * wu + c * wv;
+                }
+                for (int x = 0; x < k; ++x) {
+                    const double u = Bm[p + x * k], v = Bm[q + x * k];
+                    Bm[p + x * k] = c * u - s * v;
+                    Bm[q + x * k] = s * u + c * v;
+                }
+            }
+        if (rot == 0) break;
+    }
+    for (int b = 0; b < k; ++b) {
+        const double mu = Bm[b + b * k];
+        int rb = 0;
+        for (int a = 0; a < k; ++a) {
+            const double ma = Bm[a + a * k];
+            rb += (ma < mu) || (ma == mu && a < b);
+        }
+        eig[r0 + rb] = mu;
+        for (int a = 0; a < k; ++a) {
+            const int i = ord[r0 + a];
+            Tm[i + (long long)(r0 + rb) * n] = W[a + b * k] / sqrt(G[i + (long long)i * n]);
+        }
     }
 }
 
@@ -506,9 +508,9 @@ bool refined_generalized_eig(sdft_ctx* c, const double* M, const double* Hs, dou
     const int nmax = std::max(RE_MAX_N, std::max(n, c->nfilt));
     if (!c->reig_buf || c->reig_nmax < nmax) {
         const size_t N2 = (size_t)nmax * nmax;
-        // X, X', T, P1, P2, G, S (FP64 n x n each), ws, eig, diag, d; L / M32 / H32 (FP32); status, info
-        c->reig_buf = (double*)ctx_alloc(c, sizeof(double) * (7 * N2 + 2 * RE_KMAX * nmax + 2 * nmax + 16) +
-                                                sizeof(float) * (3 * N2 + nmax) + 64);
+        // X, X', T, P1, P2, G, S (FP64 n x n each), ws, eig, d, state; L / M32 / H32 (FP32); status, info
+        c->reig_buf = (double*)ctx_alloc(c, sizeof(double) * (7 * N2 + 2 * RE_KMAX * nmax + 2 * nmax) +
+                                                sizeof(RefineState) + sizeof(float) * (3 * N2 + nmax) + 64);
         c->reig_nmax = nmax;
     }
     const size_t N2 = (size_t)c->reig_nmax * c->reig_nmax;
@@ -522,8 +524,8 @@ bool refined_generalized_eig(sdft_ctx* c, const double* M, const double* Hs, dou
     double* ws = S + N2;
     double* ev = ws + 2 * RE_KMAX * (size_t)c->reig_nmax;
     double* dsc = ev + c->reig_nmax;
-    double* diag = dsc + c->reig_nmax;
-    float* Lg = reinterpret_cast<float*>(diag + 16);
+    RefineState* rs = reinterpret_cast<RefineState*>(dsc + c->reig_nmax);
+    float* Lg = reinterpret_cast<float*>(rs + 1);
     float* M32 = Lg + N2;
     float* H32 = M32 + N2;
     float* w32 = H32 + N2;
@@ -555,17 +557,23 @@ bool refined_generalized_eig(sdft_ctx* c, const double* M, const double* Hs, dou
         start32_kernel<<<g, 256, 0, c->stream>>>(H32, dsc, n, info, X, status);
         SDFT_CUDA(cudaGetLastError());
     }
-    const dim3 grid((n + 31) / 32, (n + 31) / 32, 2);
+    const int nt = (n + G64_T - 1) / G64_T;
+    constexpr int NT64 = G64_T * G64_T;
     for (int step = 0; step < 3; ++step) {
-        gemm64_kernel<false><<<grid, 256, 0, c->stream>>>(Prod2{{M, Hs}, {X, X}, {P1, P2}}, n, status);
-        gemm64_kernel<true><<<grid, 256, 0, c->stream>>>(Prod2{{X, X}, {P1, P2}, {G, S}}, n, status);
-        refine_step_kernel<<<1, 1024, 0, c->stream>>>(G, S, Tm, ev, ws, n, step, step == 2 ? 1 : 0, status, diag);
-        const dim3 g1(grid.x, grid.y, 1);
-        gemm64_kernel<false><<<g1, 256, 0, c->stream>>>(Prod2{{X, nullptr}, {Tm, nullptr}, {Xn, nullptr}}, n, status);
+        const int mode = step == 2 ? 1 : 0;
+        gemm64_kernel<false><<<dim3(nt, nt, 2), NT64, 0, c->stream>>>(Prod2{{M, Hs}, {X, X}, {P1, P2}}, n, status);
+        gemm64_kernel<true><<<dim3(nt, nt, 2), NT64, 0, c->stream>>>(Prod2{{X, X}, {P1, P2}, {G, S}}, n, status);
+        SDFT_CUDA(cudaMemsetAsync(rs->mx, 0, sizeof(rs->mx) + sizeof(rs->bad), c->stream));
+        refine_max_kernel<<<n, 128, 0, c->stream>>>(G, S, n, status, rs);
+        refine_order_kernel<<<1, 1024, 0, c->stream>>>(n, step, status, rs);
+        refine_fill_kernel<<<n, 128, 0, c->stream>>>(G, S, Tm, n, mode, status, rs);
+        if (mode == 1) refine_cluster_kernel<<<(n + 31) / 32, 32, 0, c->stream>>>(G, S, Tm, ev, ws, n, status, rs);
+        gemm64_kernel<false><<<dim3(nt, nt, 1), NT64, 0, c->stream>>>(Prod2{{X, nullptr}, {Tm, nullptr}, {Xn, nullptr}}, n,
+                                                                     status);
         std::swap(X, Xn);
     }
     SDFT_CUDA(cudaGetLastError());
-    count_launch(c, 13);
+    count_launch(c, 20);
     int st = 0;
     SDFT_CUDA(cudaMemcpyAsync(&st, status, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
     SDFT_CUDA(cudaStreamSynchronize(c->stream));
