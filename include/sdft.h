@@ -275,11 +275,11 @@ sdft_status sdft_rayleigh_ritz(sdft_ctx* ctx, int spin, int kpt, int precision,
  * n cells of different grids and sizes): cell i is the context ctxs[i] (SDFT_MIXED, Gamma point,
  * spin 0 V_eff as set for it), x[i] -> y[i] its FP32 paired block of nstates columns (device),
  * degree m with the cell's own bounds a0[i] < a[i] < b[i] (host arrays).  Each Chebyshev step is
- * ONE column-tile stencil launch over all cells (per-cell grid, coefficients and recurrence scalars
- * in a constant-memory table) after the cells' KB projections; every cell computes exactly what
- * sdft_chebyshev_filter computes for it with the column tile.  1 <= n <= 64; all contexts must use
+ * ONE brick-tile stencil launch over all cells (per-cell grid and coefficients in a constant-memory
+ * table) after the cells' KB projections; every cell computes exactly what
+ * sdft_chebyshev_filter computes for it with the brick tile.  1 <= n <= 64; all contexts must use
  * the same CUDA stream.  Returns after the work is enqueued and completed (synchronises).  The
- * per-cell table is ONE constant-memory array of the library, rewritten before every step: two
+ * per-cell table is ONE constant-memory array of the library, written once per call: two
  * multi-cell filters (this call or sdft_batch_scf) running at the same time on different streams or
  * host threads overwrite each other's table and give wrong results; serialise them. */
 sdft_status sdft_chebyshev_filter_multi(sdft_ctx* const* ctxs, int n, const void* const* x, void* const* y,

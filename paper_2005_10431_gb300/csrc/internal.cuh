@@ -267,6 +267,8 @@ struct sdft_ctx {
     sdft::KBProblem* g_ktab_pin = nullptr;
     sdft::KBProblem* m_ktab = nullptr;   // multi-cell filter: KB tables of every (step, cell)
     int m_ktab_cap = 0;
+    float2* m_steps = nullptr;           // multi-cell filter: (alpha, beta) of every (step, cell)
+    int m_steps_cap = 0;
     int g_pin_cap = 0;
     cudaGraphExec_t g_graph = nullptr;
     cudaStream_t cap_stream = nullptr;   // private stream for graph capture
@@ -417,8 +419,8 @@ void seed_orbitals(sdft_ctx* c, int precision, bool cplx, void* X, int ncol, uin
 int group_variant_f32(sdft_ctx* c, bool cplx, int ncolE);
 void launch_group_step_f32(sdft_ctx* c, bool cplx, int variant, const RowProblem* grp, int nprob, int ncolE,
                            bool prev, bool haskb);
-void launch_group_project_f32(sdft_ctx* c, bool cplx, const KBProblem* grp, int nprob, int ncolE);
-void launch_multi_project_f32(sdft_ctx* c, const KBProblem* grp, int nprob, int max_natom, int max_ncolE);
+// KB projections of nprob problems (device table) with at most natom atoms and ncolE columns
+void launch_group_project_f32(sdft_ctx* c, bool cplx, const KBProblem* grp, int nprob, int natom, int ncolE);
 int autotune_group_f32(sdft_ctx* c, bool cplx, const RowProblem* grp, int nprob, int ncolE, bool haskb);
 // Chebyshev filter of the FP32 real blocks of several cells (contexts with their own grids) with
 // one column-tile stencil launch per step (scf.cu; kernels in stencil_f32.cu)

@@ -476,7 +476,7 @@ static void chefsi_pass_group(sdft_ctx* c, const std::vector<Problem*>& G, int v
                                   c->stream));
         SDFT_CUDA(cudaMemcpyAsync(c->g_ktab, c->g_ktab_h.data(), sizeof(KBProblem) * ntab, cudaMemcpyHostToDevice,
                                   c->stream));
-        if (haskb) launch_group_project_f32(c, cplx, c->g_ktab + (size_t)m * np, np, ncolE);
+        if (haskb) launch_group_project_f32(c, cplx, c->g_ktab + (size_t)m * np, np, c->natom, ncolE);
         gch = autotune_group_f32(c, cplx, c->g_rtab + (size_t)m * np, np, ncolE, haskb);
     }
     if (gch >= 0) variant = gch;
@@ -485,7 +485,7 @@ static void chefsi_pass_group(sdft_ctx* c, const std::vector<Problem*>& G, int v
         SDFT_CUDA(cudaMemcpyAsync(c->g_rtab, rsrc, sizeof(RowProblem) * ntab, cudaMemcpyHostToDevice, c->stream));
         SDFT_CUDA(cudaMemcpyAsync(c->g_ktab, ksrc, sizeof(KBProblem) * ntab, cudaMemcpyHostToDevice, c->stream));
         for (int k = 0; k <= m; ++k) {
-            if (haskb) launch_group_project_f32(c, cplx, c->g_ktab + (size_t)k * np, np, ncolE);
+            if (haskb) launch_group_project_f32(c, cplx, c->g_ktab + (size_t)k * np, np, c->natom, ncolE);
             launch_group_step_f32(c, cplx, variant, c->g_rtab + (size_t)k * np, np, ncolE, k > 0 && k < m, haskb);
         }
     };

@@ -1,8 +1,7 @@
 // Instantiations of the fused stencil / Chebyshev-step kernels (see stencil_impl.cuh)
 // for FP32 blocks (two lanes per element: an orbital pair, or re/im of a Bloch orbital).
-#include "stencil_impl.cuh"
+#include "stencil_brick.cuh"
 
-#include <array>
 #include <vector>
 
 namespace sdft {
@@ -32,6 +31,9 @@ const StepVariant<float2> kReal[] = {
     {&launch_slab_variant<120, 8, 1, 1, 2, 4, 1>, &slab_variant_ok<120, 8, 1, 2, 4>, "slab120"},
     {&launch_slab_variant<40, 8, 2, 1, 2, 4, 1>, &slab_variant_ok<40, 8, 2, 2, 4>, "slab40"},
     {&launch_slab_variant<80, 8, 1, 2, 2, 4, 1>, &slab_variant_ok<80, 8, 1, 2, 4>, "slab80ry2"},
+    // bricks of 8 and 4 planes (stencil_brick.cuh)
+    {&launch_brick<float2, false, 8, 2>, &brick_ok<float2, 8>, "brick8"},
+    {&launch_brick<float2, false, 4, 2>, &brick_ok<float2, 4>, "brick4"},
 };
 const StepVariant<float2> kCplx[] = {
     {&launch_variant<float2, true, 32, 8, 2, 2, 4>, nullptr, "col32x8"},
@@ -39,10 +41,23 @@ const StepVariant<float2> kCplx[] = {
     {&launch_row_variant<true, 4, 1, 256, 2, 3>, &row_ok<4, 256, 3>, "row4", &launch_row_group<true, 4, 1, 256, 2, 3>},
     {&launch_row_variant<true, 8, 1, 256, 2, 3>, &row_ok<8, 256, 3>, "row8", &launch_row_group<true, 8, 1, 256, 2, 3>},
     {&launch_row_variant<true, 10, 1, 256, 2, 3>, &row_ok<10, 256, 3>, "row10", &launch_row_group<true, 10, 1, 256, 2, 3>},
+    {&launch_brick<float2, true, 8, 2>, &brick_ok<float2, 8>, "brick8"},
+    {&launch_brick<float2, true, 4, 2>, &brick_ok<float2, 4>, "brick4"},
 };
+constexpr int kRealBrick8 = 16, kCplxBrick8 = 5;   // the brick4 variants follow
 constexpr int kNReal = sizeof(kReal) / sizeof(kReal[0]);
 constexpr int kNCplx = sizeof(kCplx) / sizeof(kCplx[0]);
 }  // namespace
+
+// Calls too small to be timed take a brick tile: 37 x 41 x 45 points, 20 columns: 15.4 us a step, 31 with the column
+// tile; 40^3, 28 columns: 20 and 26; 48^3, 40 columns: 35 and 66.  Bricks of 8 planes need two CTAs an SM, else 4.
+static int small_variant(const sdft_ctx* c, bool cplx, int ncolE) {
+    const int v8 = cplx ? kCplxBrick8 : kRealBrick8;
+    if (!brick_ok<float2, 8>(c, ncolE)) return 0;
+    const BrickTile t = brick_tile(c->n[0], c->n[1]);
+    const long long ctas8 = (long long)t.tiles_x * t.tiles_y * ((c->n[2] + 7) / 8) * ncolE;
+    return ctas8 >= 2 * 152 ? v8 : v8 + 1;
+}
 
 template <>
 void launch_kb_project<float2>(sdft_ctx* c, int kpt, const float2* Y, float2* C, int ncolE) {
@@ -58,7 +73,11 @@ void launch_cheb_step<float2>(sdft_ctx* c, int kpt, const float2* Y, const float
     const int nvar = cplx ? kNCplx : kNReal;
     int& choice = c->stencil_choice[cplx ? 1 : 0];
     int pick = choice;
-    if (pick < 0) {
+    // the row and slab tiles move 16-byte vectors: blocks that start in between take a brick
+    const bool aligned = (((uintptr_t)Y | (uintptr_t)Yprev | (uintptr_t)Ynext) & 15) == 0;
+    if (!aligned) {
+        pick = small_variant(c, cplx, ncolE);
+    } else if (pick < 0) {
         // when the caller wants the output's KB coefficients too, the variants are timed with them (fused
         // or by the separate pass, into the caller's target buffer, which the real launch then rewrites)
         float2* kb_next = c->kb_next;
@@ -71,7 +90,7 @@ void launch_cheb_step<float2>(sdft_ctx* c, int kpt, const float2* Y, const float
             choice = pick;
             if (kb_next) c->stencil_fuse = fused;
         } else {
-            pick = 0;
+            pick = small_variant(c, cplx, ncolE);
         }
     }
     if (!c->stencil_fuse) c->kb_next = nullptr;   // the separate projection pass was timed faster
@@ -146,84 +165,102 @@ void launch_group_step_f32(sdft_ctx* c, bool cplx, int variant, const RowProblem
     table[variant].group(c, 0, grp, nprob, ncolE, prev, haskb);
 }
 
-// One column-tile launch over several cells (each its own context, grid and block); probs[i].A
-// carries cell i's recurrence step.  All contexts share the stream of the first one.
-void launch_multi_step_f32(const std::vector<sdft_ctx*>& ctxs, std::vector<MultiProblem>& probs, bool prev) {
-    constexpr int TX = 32, TY = 8, PF = 2, MINB = 2, D = 4;
-    const int n = (int)probs.size();
-    SDFT_REQUIRE(n >= 1 && n <= MULTI_MAX, SDFT_ERR_INVALID_ARG, "multi-cell launch takes 1..64 cells");
-    sdft_ctx* c0 = ctxs[0];
-    long long total = 0;
-    int max_natom = 1;
-    double bytes = 0;
-    for (int i = 0; i < n; ++i) {
-        MultiProblem& P = probs[i];
-        const sdft_ctx* c = ctxs[i];
-        P.tiles_x = (c->n[0] + TX - 1) / TX;
-        P.tiles_y = (c->n[1] + TY - 1) / TY;
-        P.cta_begin = (int)total;
-        total += (long long)P.tiles_x * P.tiles_y * (c->nfilt / 2) * P.A.nzc;
-        P.cta_end = (int)total;
-        max_natom = std::max(max_natom, c->natom);
-        bytes += (double)(c->nfilt / 2) * (double)c->ng * sizeof(float2) * (prev ? 3.0 : 2.0);
+// ---- several cells in one launch (independent grids, FP32 real blocks) --------------------
+// One cell of a multi-cell filter.  The table is written once per filter call: the blocks of step k follow from
+// the ring buffers and k, and the recurrence scalars of every (step, cell) come from a device table.
+struct MultiProblem {
+    StepArgs<float> A;                // grid, coefficients, shift
+    const float2* X;                  // the filter's input
+    float2* ring[3];                  // step k writes ring[slot(k)], see multi_slot
+    const float* V;
+    const float2* C;
+    const int* patom;
+    const void* pval;
+    int nslot, tw, th, tiles_x, cta_begin, cta_end;
+};
+__host__ __device__ inline int multi_slot(int k, int m) { return (((2 - (m - k)) % 3) + 3) % 3; }
+constexpr int MULTI_ZC = 8;
+__constant__ MultiProblem c_multi[MULTI_MAX];
+
+// step k of degree m; grid: the CTAs of every cell, cell p owning [cta_begin, cta_end) = tiles x z chunks x columns
+template <bool PREV>
+__global__ void __launch_bounds__(BRICK_NT, 2) brick_multi_kernel(const int nprob, const int k, const int m,
+                                                                 const float2* __restrict__ steps) {
+    const int b = blockIdx.x;
+    int lo = 0, hi = nprob - 1;       // the cell whose range holds b
+    while (lo < hi) {
+        const int mid = (lo + hi) >> 1;
+        if (b < c_multi[mid].cta_end) hi = mid;
+        else lo = mid + 1;
     }
-    SDFT_REQUIRE(total < (1LL << 31), SDFT_ERR_INVALID_ARG, "multi-cell launch too large");
-    SDFT_CUDA(cudaMemcpyToSymbolAsync(c_multi, probs.data(), sizeof(MultiProblem) * n, 0, cudaMemcpyHostToDevice,
-                                      c0->stream));
-    const size_t dsm = sizeof(Stage<float2, float, float, TX, TY, 3>) * D + sizeof(float2) * (size_t)max_natom;
-    ScopedTimer timer(c0, SDFT_K_STENCIL, bytes);
-    auto launch = [&](auto kfn) {
-        if (dsm > 48 * 1024)
-            SDFT_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm));
-        kfn<<<(unsigned)total, dim3(TX, TY), dsm, c0->stream>>>(n);
-    };
-    if (prev) launch(cheb_multi_kernel<TX, TY, PF, MINB, D, true>);
-    else launch(cheb_multi_kernel<TX, TY, PF, MINB, D, false>);
-    SDFT_CUDA(cudaGetLastError());
-    count_launch(c0);
-}
-
-// z chunks of one cell inside a multi-cell launch: at least 16 planes per chunk, enough CTAs overall
-int multi_nzc(const sdft_ctx* c, long long ctas_other) {
-    const long long want = 8LL * 152;
-    const long long base = (long long)((c->n[0] + 31) / 32) * ((c->n[1] + 7) / 8) * (c->nfilt / 2);
-    int nzc = 1;
-    while (ctas_other + base * nzc < want && c->n[2] / (nzc + 1) >= 16) ++nzc;
-    return nzc;
-}
-
-StepArgs<float> multi_args(sdft_ctx* c, double alpha, double beta, double shift, int nzc) {
-    const int zchunk = (c->n[2] + nzc - 1) / nzc;
-    return make_args<float>(c, 0, alpha, beta, shift, zchunk, (c->n[2] + zchunk - 1) / zchunk);
+    const MultiProblem& P = c_multi[lo];
+    int local = b - P.cta_begin;
+    const int tiles = P.tiles_x * ((P.A.n2 + P.th - 1) / P.th);
+    const int tile = local % tiles;
+    local /= tiles;
+    const int zc = local % P.A.nzc, col = local / P.A.nzc;
+    const int by = tile / P.tiles_x, bx = tile - by * P.tiles_x;
+    const float2* Y = k == 1 ? P.X : P.ring[multi_slot(k - 1, m)];
+    const float2* Yprev = k == 1 ? nullptr : (k == 2 ? P.X : P.ring[multi_slot(k - 2, m)]);
+    const float2 ab = steps[(long long)(k - 1) * nprob + lo];
+    brick_body<float2, false, MULTI_ZC, PREV, true>(Y, Yprev, P.ring[multi_slot(k, m)], P.V, P.C, P.patom, P.pval,
+                                                    P.nslot, P.A, ab.x, ab.y, P.tw, P.th, bx, by, zc * MULTI_ZC, col);
 }
 
 void chebyshev_filter_multi(const std::vector<sdft_ctx*>& ctxs, const std::vector<const void*>& X,
                             const std::vector<void*>& Y, int m, const double* a, const double* b, const double* a0) {
     const int n = (int)ctxs.size();
     SDFT_REQUIRE(m >= 1, SDFT_ERR_INVALID_ARG, "degree must be >= 1");
-    // per cell: the recurrence scalars and a ring of its own block buffers (T1, T2, Y)
-    std::vector<double> e(n), cc(n), sigma1(n), sigma(n);
-    std::vector<std::array<float2*, 3>> ring(n);
-    long long ctas = 0;
-    std::vector<int> nzc(n);
+    SDFT_REQUIRE(n >= 1 && n <= MULTI_MAX, SDFT_ERR_INVALID_ARG, "multi-cell launch takes 1..64 cells");
+    sdft_ctx* c0 = ctxs[0];
+    // per cell: grid, tile, ring of its own block buffers (T1, T2, Y), recurrence scalars of every step
+    std::vector<MultiProblem> probs(n);
+    std::vector<float2> steps((size_t)m * n);
+    long long total = 0;
+    size_t dsm = 0;
+    double elems = 0;
     for (int i = 0; i < n; ++i) {
         sdft_ctx* c = ctxs[i];
         SDFT_REQUIRE(b[i] > a[i] && a[i] > a0[i], SDFT_ERR_INVALID_ARG, "filter bounds must satisfy a0 < a < b");
-        e[i] = 0.5 * (b[i] - a[i]);
-        cc[i] = 0.5 * (b[i] + a[i]);
-        sigma1[i] = sigma[i] = e[i] / (a0[i] - cc[i]);
-        float2* t[2];
+        const double e = 0.5 * (b[i] - a[i]), cc = 0.5 * (b[i] + a[i]);
+        const double sigma1 = e / (a0[i] - cc);
+        double sigma = sigma1;
+        for (int k = 1; k <= m; ++k) {
+            double alpha = sigma1 / e, beta = 0.0;
+            if (k > 1) {
+                const double s2 = 1.0 / (2.0 / sigma1 - sigma);
+                alpha = 2.0 * s2 / e;
+                beta = sigma * s2;
+                sigma = s2;
+            }
+            steps[(size_t)(k - 1) * n + i] = make_float2((float)alpha, (float)beta);
+        }
+        MultiProblem& P = probs[i];
+        const int nzc = (c->n[2] + MULTI_ZC - 1) / MULTI_ZC;
+        P.A = make_args<float>(c, 0, 0.0, 0.0, cc, MULTI_ZC, nzc);
+        P.X = (const float2*)X[i];
         int got = 0;
         for (int k = 0; k < 4 && got < 2; ++k)
-            if (c->blk[k] != X[i] && c->blk[k] != Y[i]) t[got++] = (float2*)c->blk[k];
+            if (c->blk[k] != X[i] && c->blk[k] != Y[i]) P.ring[got++] = (float2*)c->blk[k];
         SDFT_REQUIRE(got == 2, SDFT_ERR_INVALID_ARG, "no free block buffers for the filter");
-        ring[i] = {t[0], t[1], (float2*)Y[i]};
-        nzc[i] = multi_nzc(c, ctas);
-        ctas += (long long)((c->n[0] + 31) / 32) * ((c->n[1] + 7) / 8) * (c->nfilt / 2) * nzc[i];
+        P.ring[2] = (float2*)Y[i];
+        P.V = c->veff32;
+        P.C = (const float2*)c->C32;
+        P.patom = c->kb[0].patom;
+        P.pval = c->kb[0].pval32;
+        P.nslot = c->kb[0].S;
+        const BrickTile t = brick_tile(c->n[0], c->n[1]);
+        P.tw = t.tw;
+        P.th = t.th;
+        P.tiles_x = t.tiles_x;
+        P.cta_begin = (int)total;
+        total += (long long)t.tiles_x * t.tiles_y * nzc * (c->nfilt / 2);
+        SDFT_REQUIRE(total < (1LL << 31), SDFT_ERR_INVALID_ARG, "multi-cell launch too large");
+        P.cta_end = (int)total;
+        dsm = std::max(dsm, brick_smem<float2>(t, MULTI_ZC, c->natom));
+        elems += (double)(c->nfilt / 2) * (double)c->ng;
     }
-    auto slot = [&](int i, int k) -> float2* { return ring[i][(((2 - (m - k)) % 3) + 3) % 3]; };
     // KB projections of every (step, cell): one table, uploaded once, one grouped launch per step
-    sdft_ctx* c0 = ctxs[0];
     std::vector<KBProblem> ktab;
     std::vector<int> kcell;
     int max_natom = 0, max_ncolE = 0;
@@ -235,62 +272,49 @@ void chebyshev_filter_multi(const std::vector<sdft_ctx*>& ctxs, const std::vecto
         max_ncolE = std::max(max_ncolE, ctxs[i]->nfilt / 2);
     }
     const int nk = (int)kcell.size();
-    if (nk > 0) {
-        ktab.reserve((size_t)m * nk);
-        for (int k = 1; k <= m; ++k)
-            for (int i : kcell) {
-                sdft_ctx* c = ctxs[i];
-                const KBTables& kb = c->kb[0];
-                const float2* cur = k == 1 ? (const float2*)X[i] : slot(i, k - 1);
-                ktab.push_back(KBProblem{cur, c->C32, kb.cnt, kb.idx, kb.val32, kb.gamma, kb.cap, kb.natom,
-                                         c->nfilt / 2, c->ng});
-            }
-        if (c0->m_ktab_cap < (int)ktab.size()) {
-            c0->m_ktab = (KBProblem*)ctx_alloc(c0, sizeof(KBProblem) * ktab.size());
-            c0->m_ktab_cap = (int)ktab.size();
+    ktab.reserve((size_t)m * nk);
+    for (int k = 1; k <= m; ++k)
+        for (int i : kcell) {
+            sdft_ctx* c = ctxs[i];
+            const KBTables& kb = c->kb[0];
+            const float2* cur = k == 1 ? probs[i].X : probs[i].ring[multi_slot(k - 1, m)];
+            ktab.push_back(KBProblem{cur, c->C32, kb.cnt, kb.idx, kb.val32, kb.gamma, kb.cap, kb.natom, c->nfilt / 2,
+                                     c->ng});
         }
-        // pageable source: the copy is staged before the call returns, so ktab may go out of scope
+    if (c0->m_ktab_cap < (int)ktab.size()) {
+        c0->m_ktab = (KBProblem*)ctx_alloc(c0, sizeof(KBProblem) * ktab.size());
+        c0->m_ktab_cap = (int)ktab.size();
+    }
+    if (c0->m_steps_cap < m * n) {
+        c0->m_steps = (float2*)ctx_alloc(c0, sizeof(float2) * m * n);
+        c0->m_steps_cap = m * n;
+    }
+    // pageable sources: the copies are staged before the calls return, so the vectors may go out of scope
+    if (nk > 0)
         SDFT_CUDA(cudaMemcpyAsync(c0->m_ktab, ktab.data(), sizeof(KBProblem) * ktab.size(), cudaMemcpyHostToDevice,
                                   c0->stream));
-    }
-    std::vector<MultiProblem> probs(n);
+    SDFT_CUDA(cudaMemcpyAsync(c0->m_steps, steps.data(), sizeof(float2) * steps.size(), cudaMemcpyHostToDevice,
+                              c0->stream));
+    SDFT_CUDA(cudaMemcpyToSymbolAsync(c_multi, probs.data(), sizeof(MultiProblem) * n, 0, cudaMemcpyHostToDevice,
+                                      c0->stream));
+    auto step = [&](auto kfn, int k) {
+        ScopedTimer timer(c0, SDFT_K_STENCIL, elems * sizeof(float2) * (k > 1 ? 3.0 : 2.0));
+        if (dsm > 48 * 1024)
+            SDFT_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm));
+        kfn<<<(unsigned)total, BRICK_NT, dsm, c0->stream>>>(n, k, m, c0->m_steps);
+        SDFT_CUDA(cudaGetLastError());
+        count_launch(c0);
+    };
     for (int k = 1; k <= m; ++k) {
-        if (nk > 0) launch_multi_project_f32(c0, c0->m_ktab + (size_t)(k - 1) * nk, nk, max_natom, max_ncolE);
-        for (int i = 0; i < n; ++i) {
-            sdft_ctx* c = ctxs[i];
-            const float2* cur = k == 1 ? (const float2*)X[i] : slot(i, k - 1);
-            const float2* prv = k == 1 ? nullptr : (k == 2 ? (const float2*)X[i] : slot(i, k - 2));
-            const bool kb = c->kb[0].S > 0;
-            double alpha, beta = 0.0;
-            if (k == 1) {
-                alpha = sigma1[i] / e[i];
-            } else {
-                const double s2 = 1.0 / (2.0 / sigma1[i] - sigma[i]);
-                alpha = 2.0 * s2 / e[i];
-                beta = sigma[i] * s2;
-                sigma[i] = s2;
-            }
-            MultiProblem& P = probs[i];
-            P.A = multi_args(c, alpha, beta, cc[i], nzc[i]);
-            P.Y = cur;
-            P.Yprev = prv;
-            P.Ynext = slot(i, k);
-            P.V = c->veff32;
-            P.C = (const float2*)c->C32;
-            P.patom = c->kb[0].patom;
-            P.pval = c->kb[0].pval32;
-            P.nslot = kb ? c->kb[0].S : 0;
-        }
-        launch_multi_step_f32(ctxs, probs, k > 1);
+        if (nk > 0)
+            launch_group_project_f32(c0, false, c0->m_ktab + (size_t)(k - 1) * nk, nk, max_natom, max_ncolE);
+        if (k > 1) step(brick_multi_kernel<true>, k);
+        else step(brick_multi_kernel<false>, k);
     }
 }
 
-void launch_group_project_f32(sdft_ctx* c, bool cplx, const KBProblem* grp, int nprob, int ncolE) {
-    launch_project_group_impl<float2>(c, grp, nprob, ncolE, cplx);
-}
-
-void launch_multi_project_f32(sdft_ctx* c, const KBProblem* grp, int nprob, int max_natom, int max_ncolE) {
-    launch_project_multi_impl<float2>(c, grp, nprob, max_natom, max_ncolE);
+void launch_group_project_f32(sdft_ctx* c, bool cplx, const KBProblem* grp, int nprob, int natom, int ncolE) {
+    launch_project<float2>(c, nullptr, nullptr, nullptr, natom, ncolE, nprob, cplx, grp);
 }
 
 }  // namespace sdft

@@ -1,6 +1,6 @@
 // Instantiations of the fused stencil / Chebyshev-step kernels (see stencil_impl.cuh)
 // for one element type per translation unit, so the variants compile in parallel.
-#include "stencil_impl.cuh"
+#include "stencil_brick.cuh"
 
 #include <algorithm>
 
@@ -62,6 +62,12 @@ void launch_cheb_step<double>(sdft_ctx* c, int kpt, const double* Y, const doubl
                                                              kb.pval64, kb.S, c->natom, ncolE, A);
         SDFT_CUDA(cudaGetLastError());
         count_launch(c);
+        return;
+    }
+    // The brick at every size it takes, us per step (column tile -> brick): 24^3 x 8 90 -> 16, 36^3 x 24 220 -> 125,
+    // 64^3 x 64 1487 -> 1439, 80^3 x 140 7389 -> 6081
+    if (brick_ok<double, 4>(c, ncolE) && V != nullptr) {
+        launch_brick<double, false, 4, 2>(c, kpt, Y, Yprev, Ynext, ncolE, V, kbC, alpha, beta, shift, with_kinetic, true);
         return;
     }
     launch_variant<double, false, 32, 8, 2, 1, 3>(c, kpt, Y, Yprev, Ynext, ncolE, V, kbC, alpha, beta, shift, with_kinetic,

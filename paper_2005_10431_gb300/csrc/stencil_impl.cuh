@@ -391,38 +391,6 @@ cheb_step_kernel(const E* __restrict__ Y, const E* __restrict__ Yprev, E* __rest
                                                                  blockIdx.x, blockIdx.y, blockIdx.z);
 }
 
-// ---- several grids in one launch (independent cells of uneven size, FP32 real blocks) -----
-}  // namespace
-struct MultiProblem {                 // one cell's block in a multi-grid launch of the column tile
-    StepArgs<float> A;                // grid, coefficients, recurrence step, z chunking
-    const float2* Y;
-    const float2* Yprev;
-    float2* Ynext;
-    const float* V;
-    const float2* C;
-    const int* patom;
-    const void* pval;
-    int nslot, tiles_x, tiles_y, cta_begin, cta_end;
-};
-namespace {
-__constant__ MultiProblem c_multi[MULTI_MAX];
-
-// grid: the CTAs of every problem, problem p owning [cta_begin, cta_end) (tiles_x * tiles_y * ncolE * nzc)
-template <int TX, int TY, int PF, int MINB, int D, bool PREV>
-__global__ void __launch_bounds__(TX * TY, MINB) cheb_multi_kernel(const int nprob) {
-    const int b = blockIdx.x;
-    int p = 0;
-    while (p + 1 < nprob && b >= c_multi[p].cta_end) ++p;
-    const MultiProblem& P = c_multi[p];
-    const int local = b - P.cta_begin;
-    const int bx = local % P.tiles_x;
-    const int rest = local / P.tiles_x;
-    const int by = rest % P.tiles_y;
-    const int bz = rest / P.tiles_y;
-    cheb_step_body<float2, false, TX, TY, PF, D, PREV, true, true, true>(P.Y, P.Yprev, P.Ynext, P.V, P.C, P.patom,
-                                                                          P.pval, P.nslot, P.A, bx, by, bz);
-}
-
 // ---- row-tile variant (FP32 blocks, n1 even) --------------------------------------------
 // A CTA owns TY whole x-rows (n1 points, two consecutive points per thread, one 16-byte vector)
 // and marches along z for one element-column.  Because the tile spans the full x extent, the x
@@ -705,7 +673,12 @@ cheb_row_kernel(const float2* __restrict__ Y_, const float2* __restrict__ Yprev_
     cp_async_wait<0>();
 }
 
-// KB projection: C[col][a] = gamma_a * sum_j conj(beta_a(j)) Y[idx_j, col], NC columns per CTA
+// KB projection: C[col][a] = gamma_a * sum_j conj(beta_a(j)) Y[idx_j, col], one atom and NC columns per CTA.
+// Gathers of 8- or 16-byte elements, so what counts is how many are in flight: U support points of every column
+// per pass (NC U gathers a thread) and enough CTAs, which kb_columns() arranges by the choice of NC: with eight
+// columns per CTA whatever the size, an 8-atom cell of 20 states ran 16 CTAs (20 us a projection, 4.8 now) and the
+// two-atom FP64 cell 2 (24 us, 6.0 now).  Every NC adds the points in the same order (thread t of the CTA takes points t, t + 256, ...
+// one after another, then the warp tree, then the warps), so the choice does not change a bit of the result.
 template <typename E, bool CPLX, int NC>
 __global__ void __launch_bounds__(256, 3)
 kb_project_kernel(const E* __restrict__ Y_, E* __restrict__ C_, const int* __restrict__ cnt_,
@@ -713,12 +686,14 @@ kb_project_kernel(const E* __restrict__ Y_, E* __restrict__ C_, const int* __res
                   const double* __restrict__ gamma_, int cap_, int natom, int ncolE, long long ng,
                   const KBProblem* __restrict__ grp) {
     using S = typename Elem<E>::S;
+    using KV = typename std::conditional<CPLX, E, S>::type;
+    constexpr int U0 = 128 / (NC * (int)sizeof(E)), U = U0 < 1 ? 1 : (U0 > 8 ? 8 : U0);   // 128 bytes of Y in flight
     // one problem, or (grp != null) problem blockIdx.z of a grouped launch
     const E* __restrict__ Y = Y_;
     E* __restrict__ C = C_;
     const int* __restrict__ cnt = cnt_;
     const int* __restrict__ idx = idx_;
-    const void* __restrict__ val = val_;
+    const KV* __restrict__ val = reinterpret_cast<const KV*>(val_);
     const double* __restrict__ gamma = gamma_;
     int cap = cap_;
     if (grp) {
@@ -727,7 +702,7 @@ kb_project_kernel(const E* __restrict__ Y_, E* __restrict__ C_, const int* __res
         C = reinterpret_cast<E*>(P.C);
         cnt = P.cnt;
         idx = P.idx;
-        val = P.val;
+        val = reinterpret_cast<const KV*>(P.val);
         gamma = P.gamma;
         cap = P.cap;
         natom = P.natom;
@@ -738,51 +713,45 @@ kb_project_kernel(const E* __restrict__ Y_, E* __restrict__ C_, const int* __res
     const int c0 = blockIdx.y * NC;
     if (a >= natom || c0 >= ncolE) return;   // grouped launch sized for the largest problem
     const int m = cnt[a];
+    idx += (long long)a * cap;
+    val += (long long)a * cap;
+    const E* __restrict__ col[NC];           // columns past the block read its last one and are not written
+#pragma unroll
+    for (int k = 0; k < NC; ++k) col[k] = Y + (long long)min(c0 + k, ncolE - 1) * ng;
     E acc[NC];
 #pragma unroll
     for (int k = 0; k < NC; ++k) acc[k] = ezero<E>();
-    // two projector points per pass (2 NC independent gathers in flight per thread); the points of
-    // one thread are summed in the same order as one at a time
-    auto add_point = [&](long long e, int g) {
+    auto add = [&](KV b, const E* y) {
 #pragma unroll
         for (int k = 0; k < NC; ++k) {
-            if (c0 + k < ncolE) {
-                E y = Y[(long long)(c0 + k) * ng + g];
-                if constexpr (CPLX) {
-                    E b = reinterpret_cast<const E*>(val)[e];
-                    acc[k] = eadd(acc[k], cmul_conj(b, y));
-                } else {
-                    S b = reinterpret_cast<const S*>(val)[e];
-                    acc[k] = efma(b, y, acc[k]);
-                }
-            }
+            if constexpr (CPLX) acc[k] = eadd(acc[k], cmul_conj(b, y[k]));
+            else acc[k] = efma(b, y[k], acc[k]);
         }
     };
     int j = threadIdx.x;
-    for (; j + (int)blockDim.x < m; j += 2 * blockDim.x) {
-        const long long e0 = (long long)a * cap + j, e1 = e0 + blockDim.x;
-        const int g0 = idx[e0], g1 = idx[e1];
-        E y0[NC], y1[NC];
+    for (; j + (U - 1) * 256 < m; j += U * 256) {
+        int g[U];
+        KV b[U];
+        E y[U][NC];
 #pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            const bool in = c0 + k < ncolE;
-            y0[k] = in ? Y[(long long)(c0 + k) * ng + g0] : ezero<E>();
-            y1[k] = in ? Y[(long long)(c0 + k) * ng + g1] : ezero<E>();
+        for (int u = 0; u < U; ++u) g[u] = idx[j + u * 256];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            b[u] = val[j + u * 256];
+#pragma unroll
+            for (int k = 0; k < NC; ++k) y[u][k] = col[k][g[u]];
         }
 #pragma unroll
-        for (int k = 0; k < NC; ++k) {
-            if constexpr (CPLX) {
-                const E b0 = reinterpret_cast<const E*>(val)[e0], b1 = reinterpret_cast<const E*>(val)[e1];
-                acc[k] = eadd(acc[k], cmul_conj(b0, y0[k]));
-                acc[k] = eadd(acc[k], cmul_conj(b1, y1[k]));
-            } else {
-                const S b0 = reinterpret_cast<const S*>(val)[e0], b1 = reinterpret_cast<const S*>(val)[e1];
-                acc[k] = efma(b0, y0[k], acc[k]);
-                acc[k] = efma(b1, y1[k], acc[k]);
-            }
-        }
+        for (int u = 0; u < U; ++u) add(b[u], y[u]);
     }
-    if (j < m) add_point((long long)a * cap + j, idx[(long long)a * cap + j]);
+    for (; j < m; j += 256) {
+        const int g = idx[j];
+        const KV b = val[j];
+        E y[NC];
+#pragma unroll
+        for (int k = 0; k < NC; ++k) y[k] = col[k][g];
+        add(b, y);
+    }
     // block reduction (warp shuffles, then smem across warps)
     __shared__ E red[NC][8];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -805,7 +774,7 @@ kb_project_kernel(const E* __restrict__ Y_, E* __restrict__ C_, const int* __res
     if (threadIdx.x < NC && c0 + (int)threadIdx.x < ncolE) {
         const int k = threadIdx.x;
         E v = red[k][0];
-        for (int w = 1; w < (int)(blockDim.x >> 5); ++w) v = eadd(v, red[k][w]);
+        for (int w = 1; w < 8; ++w) v = eadd(v, red[k][w]);
         const S gm = (S)gamma[a];
         E out = efma(gm, v, ezero<E>());
         C[(long long)(c0 + k) * natom + a] = out;
@@ -1043,35 +1012,37 @@ int autotune_stencil(sdft_ctx* c, const StepVariant<E>* table, int nvar, int kpt
 
 }  // namespace
 
-template <typename E>
-void launch_project_group_impl(sdft_ctx* c, const KBProblem* grp, int nprob, int ncolE, bool cplx) {
-    const int natom = c->natom;
-    if (natom == 0 || ncolE == 0 || nprob == 0) return;
-    constexpr int NC = 8;
-    dim3 grid(natom, (ncolE + NC - 1) / NC, nprob);
-    ScopedTimer timer(c, SDFT_K_KB_PROJECT);
-    if (cplx) {
-        if constexpr (!std::is_same<E, double>::value)
-            kb_project_kernel<E, true, NC><<<grid, 256, 0, c->stream>>>(nullptr, nullptr, nullptr, nullptr, nullptr,
-                                                                       nullptr, 0, natom, ncolE, c->ng, grp);
-    } else {
-        kb_project_kernel<E, false, NC><<<grid, 256, 0, c->stream>>>(nullptr, nullptr, nullptr, nullptr, nullptr,
-                                                                    nullptr, 0, natom, ncolE, c->ng, grp);
-    }
-    SDFT_CUDA(cudaGetLastError());
-    count_launch(c);
+// Columns per CTA of a projection over `nprob` problems: two, or one where two leave SMs without a CTA.  Measured, us
+// per projection with 8 columns before (two points per pass) and with 8, 4, 2, 1 now: 216 atoms, 260 pairs 572 and
+// 582, 599, 549, 563; 64 atoms, 90 pairs 84.5 and 72, 73, 71, 71; 16 atoms, 20 pairs (48^3) 18.6, 11.2, 10.9, 9.3;
+// 8 atoms, 14 pairs (40^3) 17.1, 10.6, 9.7, 8.3.
+inline int kb_columns(int natom, int ncolE, int nprob) {
+    return (long long)natom * ((ncolE + 1) / 2) * nprob < 2 * 152 ? 1 : 2;
 }
 
-// one launch over problems of different sizes (cells of a multi-cell filter): grid sized for the
-// largest, blocks past a problem's atoms or columns return at once
+// projections of one problem (T) or of nprob problems of at most natom atoms and ncolE columns (grp: device table)
 template <typename E>
-void launch_project_multi_impl(sdft_ctx* c, const KBProblem* grp, int nprob, int max_natom, int max_ncolE) {
-    if (max_natom == 0 || max_ncolE == 0 || nprob == 0) return;
-    constexpr int NC = 8;
-    dim3 grid(max_natom, (max_ncolE + NC - 1) / NC, nprob);
+void launch_project(sdft_ctx* c, const E* Y, E* C, const KBTables* T, int natom, int ncolE, int nprob, bool cplx,
+                    const KBProblem* grp) {
+    if (natom == 0 || ncolE == 0 || nprob == 0) return;
     ScopedTimer timer(c, SDFT_K_KB_PROJECT);
-    kb_project_kernel<E, false, NC><<<grid, 256, 0, c->stream>>>(nullptr, nullptr, nullptr, nullptr, nullptr, nullptr,
-                                                                0, 0, 0, 0, grp);
+    using S = typename Elem<E>::S;
+    const void* val = T ? (std::is_same<S, float>::value ? (const void*)T->val32 : (const void*)T->val64) : nullptr;
+    auto launch = [&](auto kfn, int nc) {
+        kfn<<<dim3(natom, (ncolE + nc - 1) / nc, nprob), 256, 0, c->stream>>>(
+            Y, C, T ? T->cnt : nullptr, T ? T->idx : nullptr, val, T ? T->gamma : nullptr, T ? T->cap : 0, natom,
+            ncolE, c->ng, grp);
+    };
+    auto pick = [&](auto cp) {
+        constexpr bool CP = decltype(cp)::value;
+        if (kb_columns(natom, ncolE, nprob) == 2) launch(kb_project_kernel<E, CP, 2>, 2);
+        else launch(kb_project_kernel<E, CP, 1>, 1);
+    };
+    if (cplx) {
+        if constexpr (!std::is_same<E, double>::value) pick(std::true_type());
+    } else {
+        pick(std::false_type());
+    }
     SDFT_CUDA(cudaGetLastError());
     count_launch(c);
 }
@@ -1079,22 +1050,7 @@ void launch_project_multi_impl(sdft_ctx* c, const KBProblem* grp, int nprob, int
 template <typename E>
 void launch_project_impl(sdft_ctx* c, int kpt, const E* Y, E* C, int ncolE) {
     const KBTables& kb = c->kb[kpt];
-    if (kb.natom == 0 || ncolE == 0) return;
-    constexpr int NC = 8;
-    dim3 grid(kb.natom, (ncolE + NC - 1) / NC);
-    ScopedTimer timer(c, SDFT_K_KB_PROJECT);
-    using S = typename Elem<E>::S;
-    const void* val = std::is_same<S, float>::value ? (const void*)kb.val32 : (const void*)kb.val64;
-    if (kb.cplx) {
-        if constexpr (!std::is_same<E, double>::value)
-            kb_project_kernel<E, true, NC><<<grid, 256, 0, c->stream>>>(Y, C, kb.cnt, kb.idx, val, kb.gamma,
-                                                                       kb.cap, kb.natom, ncolE, c->ng, nullptr);
-    } else {
-        kb_project_kernel<E, false, NC><<<grid, 256, 0, c->stream>>>(Y, C, kb.cnt, kb.idx, val, kb.gamma, kb.cap,
-                                                                    kb.natom, ncolE, c->ng, nullptr);
-    }
-    SDFT_CUDA(cudaGetLastError());
-    count_launch(c);
+    launch_project<E>(c, Y, C, &kb, kb.natom, ncolE, 1, kb.cplx, nullptr);
 }
 
 }  // namespace sdft
