@@ -20,16 +20,36 @@ struct AtomG {
 // ---------------------------------------------------------------------------------------
 // reductions: deterministic two-stage sums of several dot products
 // ---------------------------------------------------------------------------------------
+struct DotArgs {
+    const double* a[8];
+    const double* b[8];
+};
+// K dots at once; the pointers come with the launch (no table upload), the K accumulators in registers
 template <int K>
-__global__ void multidot_kernel(const double* const* __restrict__ A, const double* const* __restrict__ B, long long n,
-                                double* __restrict__ part) {
+__global__ void __launch_bounds__(RB) multidot_kernel(const __grid_constant__ DotArgs P, long long n,
+                                                      double* __restrict__ part) {
     double acc[K];
 #pragma unroll
     for (int k = 0; k < K; ++k) acc[k] = 0.0;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+    const long long step = (long long)gridDim.x * blockDim.x;
+    long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
+    for (; i + 3 * step < n; i += 4 * step) {   // four points' loads in flight, added in order
+        double x[4][K], y[4][K];
 #pragma unroll
-        for (int k = 0; k < K; ++k)
-            if (A[k]) acc[k] = fma(A[k][i], B[k][i], acc[k]);
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int k = 0; k < K; ++k) {
+                x[u][k] = P.a[k][i + u * step];
+                y[u][k] = P.b[k][i + u * step];
+            }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+#pragma unroll
+            for (int k = 0; k < K; ++k) acc[k] = fma(x[u][k], y[u][k], acc[k]);
+    }
+    for (; i < n; i += step) {
+#pragma unroll
+        for (int k = 0; k < K; ++k) acc[k] = fma(P.a[k][i], P.b[k][i], acc[k]);
     }
     __shared__ double sh[K][RB / 32];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -47,13 +67,24 @@ __global__ void multidot_kernel(const double* const* __restrict__ A, const doubl
     }
 }
 
-template <int K>
-__global__ void multidot_finish_kernel(const double* __restrict__ part, int nblk, double* __restrict__ out) {
+// v + x[0] + x[stride] + ... (count terms, added one after another with `U` loads in flight)
+template <int U>
+__device__ __forceinline__ double ordered_sum(const double* __restrict__ x, int count, long long stride, double v = 0.0) {
+    int s = 0;
+    for (; s + U <= count; s += U) {
+        double t[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) t[u] = x[(s + u) * stride];
+#pragma unroll
+        for (int u = 0; u < U; ++u) v += t[u];
+    }
+    for (; s < count; ++s) v += x[s * stride];
+    return v;
+}
+
+__global__ void multidot_finish_kernel(const double* __restrict__ part, int nblk, int K, double* __restrict__ out) {
     const int k = threadIdx.x;
-    if (k >= K) return;
-    double v = 0.0;
-    for (int b = 0; b < nblk; ++b) v += part[(long long)b * K + k];
-    out[k] = v;
+    if (k < K) out[k] = ordered_sum<32>(part + k, nblk, K);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -180,11 +211,60 @@ __global__ void anderson_update_kernel(T* __restrict__ x, const T* __restrict__ 
     }
 }
 
+// Sum each of ND per-thread values over the CTA into row[0..ND), with sh[ND][NW] of scratch.  32 values at a
+// time are reduced together: at each of the five levels a lane keeps one half of its values and adds the partner
+// lane's, so 31 additions serve 32 values where one shuffle tree per value takes 160 (FP64 additions are what such
+// a reduction costs on this GPU).  The pairs added are the tree's (lane l with l + 16, then + 8, ...), so the sums
+// are the same bit for bit.
+template <int ND, int NW>
+__device__ __forceinline__ void block_sum(const double* vals, double* __restrict__ row, double (*sh)[NW]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k0 = 0; k0 < ND; k0 += 32) {
+        const int left = ND - k0;
+        if (left >= 6) {   // fewer values: one tree each is as cheap
+            double w[32];
+#pragma unroll
+            for (int k = 0; k < 32; ++k) w[k] = k < left ? vals[k0 + k < ND ? k0 + k : 0] : 0.0;
+#pragma unroll
+            for (int off = 16; off > 0; off >>= 1) {
+                const bool up = (lane & off) != 0;
+#pragma unroll
+                for (int k = 0; k < off; ++k) {
+                    if (k < left) {   // values past ND are never kept
+                        const double send = up ? w[k] : w[k + off];
+                        const double keep = up ? w[k + off] : w[k];
+                        w[k] = keep + __shfl_xor_sync(0xffffffffu, send, off);
+                    }
+                }
+            }
+            if (lane < left) sh[k0 + lane][warp] = w[0];
+        } else {
+#pragma unroll
+            for (int k = 0; k < 6; ++k) {
+                if (k < left) {
+                    double v = vals[k0 + k < ND ? k0 + k : 0];
+                    for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
+                    if (lane == 0) sh[k0 + k][warp] = v;
+                }
+            }
+        }
+    }
+    __syncthreads();
+    for (int k = threadIdx.x; k < ND; k += blockDim.x) {
+        double v = 0.0;
+        for (int w = 0; w < NW; ++w) v += sh[k][w];
+        row[k] = v;
+    }
+}
+
 // Gram of the history: G[i][j] = F_i . F_j (i <= j), r_i = F_i . (c f), plus f.f, for points
-// [lo, hi) strided by `step`; C = history length at compile time keeps the accumulators in registers.
-template <int C, typename T>
+// [lo, hi) strided by `step`, summed over the CTA into row; C = history length at compile time keeps the
+// accumulators in registers.
+template <int C, int NW, typename T>
 __device__ __forceinline__ void gram_accum(const T* __restrict__ F, const int* sl, const T* __restrict__ f, T c,
-                                           long long n, long long lo, long long hi, long long step, double* out) {
+                                           long long n, long long lo, long long hi, long long step, double* row,
+                                           double (*sh)[NW]) {
     constexpr int ND = C * (C + 1) / 2 + C + 1;
     T acc[ND];
 #pragma unroll
@@ -203,39 +283,24 @@ __device__ __forceinline__ void gram_accum(const T* __restrict__ F, const int* s
         for (int a = 0; a < C; ++a) acc[k++] += v[a] * fi;
         acc[k] += fi * fi;
     }
+    double out[ND];
 #pragma unroll
     for (int k = 0; k < ND; ++k) out[k] = (double)acc[k];
+    block_sum<ND, NW>(out, row, sh);
 }
 
-// per-thread partials of the history Gram for a runtime history length m <= 16
-template <typename T>
+// the CTA's partial history Gram for a runtime history length m <= 16
+template <int NW, typename T>
 __device__ void gram_accum_dispatch(int m, const T* F, const int* sl, const T* f, T c, long long n, long long lo,
-                                    long long hi, long long step, double* out) {
+                                    long long hi, long long step, double* row, double (*sh)[NW]) {
     switch (m) {
 #define SDFT_GRAM_CASE(CC) \
-    case CC: gram_accum<CC, T>(F, sl, f, c, n, lo, hi, step, out); break;
+    case CC: gram_accum<CC, NW, T>(F, sl, f, c, n, lo, hi, step, row, sh); break;
         SDFT_GRAM_CASE(0) SDFT_GRAM_CASE(1) SDFT_GRAM_CASE(2) SDFT_GRAM_CASE(3) SDFT_GRAM_CASE(4) SDFT_GRAM_CASE(5)
         SDFT_GRAM_CASE(6) SDFT_GRAM_CASE(7) SDFT_GRAM_CASE(8) SDFT_GRAM_CASE(9) SDFT_GRAM_CASE(10) SDFT_GRAM_CASE(11)
         SDFT_GRAM_CASE(12) SDFT_GRAM_CASE(13) SDFT_GRAM_CASE(14) SDFT_GRAM_CASE(15) SDFT_GRAM_CASE(16)
 #undef SDFT_GRAM_CASE
         default: break;
-    }
-}
-
-// block-reduce nd per-thread values (in `vals`, one per thread slot) into part[blockIdx.x * nd + k]
-template <int NW>
-__device__ void block_reduce_partials(const double* vals, int nd, double* part_row, double (*sh)[NW]) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int k = 0; k < nd; ++k) {
-        double v = vals[k];
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_down_sync(0xffffffffu, v, off);
-        if (lane == 0) sh[k][warp] = v;
-    }
-    __syncthreads();
-    for (int k = threadIdx.x; k < nd; k += blockDim.x) {
-        double v = 0.0;
-        for (int w = 0; w < NW; ++w) v += sh[k][w];
-        part_row[k] = v;
     }
 }
 
@@ -248,61 +313,91 @@ __global__ void __launch_bounds__(RB) anderson_gram_kernel(const T* __restrict__
     __shared__ double sh[GRAM_MAXND][RB / 32];
     int sl[16];
     for (int j = 0; j < m; ++j) sl[j] = slots[j];
-    double vals[GRAM_MAXND];
     const long long step = (long long)gridDim.x * blockDim.x;
-    gram_accum_dispatch<T>(m, F, sl, f, c, n, blockIdx.x * (long long)blockDim.x + threadIdx.x, n, step, vals);
     const int nd = m * (m + 1) / 2 + m + 1;
-    block_reduce_partials<RB / 32>(vals, nd, part + (long long)blockIdx.x * nd, sh);
+    gram_accum_dispatch<RB / 32, T>(m, F, sl, f, c, n, blockIdx.x * (long long)blockDim.x + threadIdx.x, n, step,
+                                    part + (long long)blockIdx.x * nd, sh);
 }
 
-// sum partials (one thread per entry, in block order), then solve (F^T F) gamma = F^T f by
-// Gaussian elimination with partial pivoting on one thread
+// two at once: blockIdx.y 0 the history Gram with f, blockIdx.y 1 the norm of g
+template <typename T>
+__global__ void __launch_bounds__(RB) anderson_gram2_kernel(const T* __restrict__ F, const int* __restrict__ slots, int m,
+                                                            const T* __restrict__ f, const T* __restrict__ g, T c,
+                                                            long long n, double* __restrict__ part,
+                                                            double* __restrict__ part_g) {
+    __shared__ double sh[GRAM_MAXND][RB / 32];
+    int sl[16];
+    const int mm = blockIdx.y == 0 ? m : 0, nd = mm * (mm + 1) / 2 + mm + 1;
+    for (int j = 0; j < mm; ++j) sl[j] = slots[j];
+    gram_accum_dispatch<RB / 32, T>(mm, F, sl, blockIdx.y == 0 ? f : g, c, n,
+                                    blockIdx.x * (long long)blockDim.x + threadIdx.x, n,
+                                    (long long)gridDim.x * blockDim.x,
+                                    (blockIdx.y == 0 ? part : part_g) + (long long)blockIdx.x * nd, sh);
+}
+
+// sum partials (one thread per entry, in block order), then solve (F^T F) gamma = F^T f by Gaussian elimination
+// with partial pivoting in the first warp: the rows' factors by one lane each, then every (row, column) update by
+// its own lane (one thread through a matrix in local memory took 25 us for m = 7, 14.7 us now)
 __device__ void anderson_solve_block(const double* __restrict__ part, int nblk, int m, double* gamma, double* ff) {
     __shared__ double s[GRAM_MAXND];
+    __shared__ double G[16][17], x[16];
     const int nd = m * (m + 1) / 2 + m + 1;
-    for (int k = threadIdx.x; k < nd; k += blockDim.x) {
-        double v = 0.0;
-        for (int b = 0; b < nblk; ++b) v += part[(long long)b * nd + k];
-        s[k] = v;
-    }
+    for (int k = threadIdx.x; k < nd; k += blockDim.x) s[k] = ordered_sum<16>(part + k, nblk, nd);
     __syncthreads();
-    if (threadIdx.x != 0) return;
-    double G[16][17];
-    int k = 0;
-    for (int a = 0; a < m; ++a)
-        for (int b = a; b < m; ++b) {
-            G[a][b] = s[k];
-            G[b][a] = s[k];
-            ++k;
-        }
-    for (int a = 0; a < m; ++a) G[a][m] = s[k++];
-    *ff = s[k];
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x;
+    if (lane == 0) *ff = s[nd - 1];
+    for (int e = lane; e < m * m; e += 32) {
+        const int a = e / m, b = e - a * m, lo = min(a, b), hi = max(a, b);
+        G[a][b] = s[lo * m - lo * (lo - 1) / 2 + hi - lo];
+    }
+    for (int a = lane; a < m; a += 32) G[a][m] = s[m * (m + 1) / 2 + a];
+    __syncwarp();
     for (int col = 0; col < m; ++col) {
         int piv = col;
         for (int r = col + 1; r < m; ++r)
             if (fabs(G[r][col]) > fabs(G[piv][col])) piv = r;
-        if (piv != col)
-            for (int q = 0; q <= m; ++q) {
-                const double t = G[col][q];
-                G[col][q] = G[piv][q];
-                G[piv][q] = t;
-            }
+        __syncwarp();
+        if (piv != col && lane <= m) {
+            const double t = G[col][lane];
+            G[col][lane] = G[piv][lane];
+            G[piv][lane] = t;
+        }
+        __syncwarp();
         const double d = G[col][col];
-        for (int r = col + 1; r < m; ++r) {
-            const double fct = d != 0.0 ? G[r][col] / d : 0.0;
-            for (int q = col; q <= m; ++q) G[r][q] -= fct * G[col][q];
+        const double fct = lane > col && lane < m && d != 0.0 ? G[lane][col] / d : 0.0;   // row `lane`
+        __syncwarp();
+        const int w = m + 1 - col, rows = m - 1 - col;
+        for (int e0 = 0; e0 < rows * w; e0 += 32) {
+            const int e = e0 + lane, i = e / w, q = col + e - i * w, r = col + 1 + i;
+            const double f = __shfl_sync(0xffffffffu, fct, r & 31);
+            if (e < rows * w) G[r][q] -= f * G[col][q];
+        }
+        __syncwarp();
+    }
+    // back substitution, row by row; a row subtracts its known terms in ascending column order
+    for (int r = m - 1; r >= 0; --r) {
+        if (lane == 0) {
+            double v = G[r][m];
+            for (int q = r + 1; q < m; ++q) v -= G[r][q] * x[q];
+            x[r] = G[r][r] != 0.0 ? v / G[r][r] : 0.0;
         }
     }
-    for (int r = m - 1; r >= 0; --r) {
-        double v = G[r][m];
-        for (int q = r + 1; q < m; ++q) v -= G[r][q] * gamma[q];
-        gamma[r] = G[r][r] != 0.0 ? v / G[r][r] : 0.0;
-    }
+    __syncwarp();
+    if (lane < m) gamma[lane] = x[lane];
 }
 
 __global__ void anderson_solve_kernel(const double* __restrict__ part, int nblk, int m, double* __restrict__ gamma,
                                       double* __restrict__ ff) {
     anderson_solve_block(part, nblk, m, gamma, ff);
+}
+
+// blockIdx.x 0: solve the history Gram in part; 1: sum the norm's partials into *rr
+__global__ void anderson_solve2_kernel(const double* __restrict__ part, const double* __restrict__ part_g, int nblk,
+                                       int m, double* __restrict__ gamma, double* __restrict__ ff,
+                                       double* __restrict__ rr) {
+    if (blockIdx.x == 0) anderson_solve_block(part, nblk, m, gamma, ff);
+    else anderson_solve_block(part_g, nblk, 0, nullptr, rr);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -676,25 +771,29 @@ std::vector<AtomG> atom_g(sdft_ctx* c) {
 // out[k] = a_k . b_k for k < count (<= 8), synchronously to host
 void dots_host(sdft_ctx* c, int count, const double* const* a, const double* const* b, long long n, double* host_out) {
     SDFT_REQUIRE(count >= 1 && count <= 8, SDFT_ERR_INVALID_ARG, "dots_host: count");
-    const double* pa[8] = {nullptr};
-    const double* pb[8] = {nullptr};
+    DotArgs P{};
     for (int k = 0; k < count; ++k) {
-        pa[k] = a[k];
-        pb[k] = b[k];
+        P.a[k] = a[k];
+        P.b[k] = b[k];
     }
-    // pointer tables live in the small scalar area
-    const double** dA = (const double**)(c->scal + 1024);
-    const double** dB = (const double**)(c->scal + 1024 + 8);
     double* part = c->scal + 2048;
     double* out = c->scal + 1536;
-    SDFT_CUDA(cudaMemcpyAsync((void*)dA, pa, sizeof(pa), cudaMemcpyHostToDevice, c->stream));
-    SDFT_CUDA(cudaMemcpyAsync((void*)dB, pb, sizeof(pb), cudaMemcpyHostToDevice, c->stream));
     const int nblk = 128;  // 128 blocks x 8 dots fits in the 2048-double partial area
-    multidot_kernel<8><<<nblk, RB, 0, c->stream>>>(dA, dB, n, part);
-    multidot_finish_kernel<8><<<1, 32, 0, c->stream>>>(part, nblk, out);
+    auto launch = [&](auto kfn) { kfn<<<nblk, RB, 0, c->stream>>>(P, n, part); };
+    switch (count) {
+        case 1: launch(multidot_kernel<1>); break;
+        case 2: launch(multidot_kernel<2>); break;
+        case 3: launch(multidot_kernel<3>); break;
+        case 4: launch(multidot_kernel<4>); break;
+        case 5: launch(multidot_kernel<5>); break;
+        case 6: launch(multidot_kernel<6>); break;
+        case 7: launch(multidot_kernel<7>); break;
+        default: launch(multidot_kernel<8>); break;
+    }
+    multidot_finish_kernel<<<1, 32, 0, c->stream>>>(part, nblk, count, out);
     SDFT_CUDA(cudaGetLastError());
     count_launch(c, 2);
-    SDFT_CUDA(cudaMemcpyAsync(c->hscal, out, sizeof(double) * 8, cudaMemcpyDeviceToHost, c->stream));
+    SDFT_CUDA(cudaMemcpyAsync(c->hscal, out, sizeof(double) * count, cudaMemcpyDeviceToHost, c->stream));
     SDFT_CUDA(cudaStreamSynchronize(c->stream));
     for (int k = 0; k < count; ++k) host_out[k] = c->hscal[k];
 }
@@ -881,26 +980,38 @@ void veff_to_float(sdft_ctx* c, int spin) {
 // point with direct neighbour loads: the vector is a few MB and stays in L2, so a flat grid of
 // short independent threads beats the z-marching tile kernel built for orbital blocks.
 // ---------------------------------------------------------------------------------------
-struct LapCoef {
-    double c[3][FD_RADIUS + 1];  // -1/2 w_r / h_d^2
-    double c0;
-};
-
 template <typename T>
-__global__ void __launch_bounds__(256) laplacian_residual_kernel(const T* __restrict__ x, const T* __restrict__ b,
-                                                                 T* __restrict__ out, LapCoef K, int n1, int n2,
-                                                                 int n3, T shift, int dirichlet) {
+struct LapCoefT {        // in the vector's own type: converting on use would cost an FP64-rate instruction each
+    T c[3][FD_RADIUS + 1];  // -1/2 w_r / h_d^2
+    T c0;
+};
+using LapCoef = LapCoefT<double>;
+template <typename T>
+LapCoefT<T> lap_coef(const sdft_ctx* c) {
+    LapCoefT<T> K;
+    for (int r = 0; r <= FD_RADIUS; ++r) {
+        K.c[0][r] = (T)c->coef.cx[r];
+        K.c[1][r] = (T)c->coef.cy[r];
+        K.c[2][r] = (T)c->coef.cz[r];
+    }
+    K.c0 = (T)c->coef.c0;
+    return K;
+}
+
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+
+template <typename T, bool DIR>
+__device__ __forceinline__ T laplacian_residual_at(const T* __restrict__ x, const T* __restrict__ b, const LapCoefT<T>& K,
+                                                   int n1, int n2, int n3, T shift, int g) {
     // 32-bit indices: the grid has < 2^31 points
     const int plane = n1 * n2;
-    const int ng = plane * n3;
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= ng) return;
     const int k = g / plane;
     const int rem = g - k * plane;
     const int j = rem / n1;
     const int i = rem - j * n1;
     const int row = g - i, col = g - j * n1, pl = g - k * plane;
-    T acc = (T)K.c0 * x[g];
+    T acc = mul_rn(K.c0, x[g]);   // roundings spelled out: a contraction of the first terms would change the sum
 #pragma unroll
     for (int r = 1; r <= FD_RADIUS; ++r) {
         int ip = i + r, im = i - r, jp = j + r, jm = j - r, kp = k + r, km = k - r;
@@ -910,31 +1021,76 @@ __global__ void __launch_bounds__(256) laplacian_residual_kernel(const T* __rest
         jm += jm < 0 ? n2 : 0;
         kp -= kp >= n3 ? n3 : 0;
         km += km < 0 ? n3 : 0;
-        if (dirichlet) {   // zero beyond the grid (isolated systems: ghost values enter through b)
-            acc += (T)K.c[0][r] * ((i + r < n1 ? x[row + ip] : (T)0) + (i - r >= 0 ? x[row + im] : (T)0));
-            acc += (T)K.c[1][r] * ((j + r < n2 ? x[col + jp * n1] : (T)0) + (j - r >= 0 ? x[col + jm * n1] : (T)0));
-            acc += (T)K.c[2][r] * ((k + r < n3 ? x[pl + kp * plane] : (T)0) + (k - r >= 0 ? x[pl + km * plane] : (T)0));
+        if (DIR) {   // zero beyond the grid (isolated systems: ghost values enter through b)
+            acc = fma(K.c[0][r], (i + r < n1 ? x[row + ip] : (T)0) + (i - r >= 0 ? x[row + im] : (T)0), acc);
+            acc = fma(K.c[1][r], (j + r < n2 ? x[col + jp * n1] : (T)0) + (j - r >= 0 ? x[col + jm * n1] : (T)0), acc);
+            acc = fma(K.c[2][r], (k + r < n3 ? x[pl + kp * plane] : (T)0) + (k - r >= 0 ? x[pl + km * plane] : (T)0), acc);
         } else {
-            acc += (T)K.c[0][r] * (x[row + ip] + x[row + im]);
-            acc += (T)K.c[1][r] * (x[col + jp * n1] + x[col + jm * n1]);
-            acc += (T)K.c[2][r] * (x[pl + kp * plane] + x[pl + km * plane]);
+            acc = fma(K.c[0][r], x[row + ip] + x[row + im], acc);
+            acc = fma(K.c[1][r], x[col + jp * n1] + x[col + jm * n1], acc);
+            acc = fma(K.c[2][r], x[pl + kp * plane] + x[pl + km * plane], acc);
         }
     }
-    // -L x = 2 * (-1/2 L x): out = b + L x - shift x = b - 2 acc - shift x  (residual of (-L + shift) x = b)
-    out[g] = b[g] - (T)2 * acc - shift * x[g];
+    // -L x = 2 * (-1/2 L x): b + L x - shift x = b - 2 acc - shift x  (residual of (-L + shift) x = b)
+    return fma(-shift, x[g], fma((T)-2, acc, b[g]));
+}
+
+template <typename T, bool DIR>
+__global__ void __launch_bounds__(256) laplacian_residual_kernel(const T* __restrict__ x, const T* __restrict__ b,
+                                                                 T* __restrict__ out,
+                                                                 const __grid_constant__ LapCoefT<T> K, int n1, int n2,
+                                                                 int n3, T shift) {
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g < n1 * n2 * n3) out[g] = laplacian_residual_at<T, DIR>(x, b, K, n1, n2, n3, shift, g);
 }
 
 template <typename T>
 void laplacian_residual(sdft_ctx* c, const T* x, const T* b, T* out, T shift = T(0)) {
-    LapCoef K;
-    for (int r = 0; r <= FD_RADIUS; ++r) {
-        K.c[0][r] = c->coef.cx[r];
-        K.c[1][r] = c->coef.cy[r];
-        K.c[2][r] = c->coef.cz[r];
+    const LapCoefT<T> K = lap_coef<T>(c);
+    auto launch = [&](auto kfn) {
+        kfn<<<(unsigned)((c->ng + 255) / 256), 256, 0, c->stream>>>(x, b, out, K, c->n[0], c->n[1], c->n[2], shift);
+    };
+    if (c->opt.boundary == SDFT_BC_DIRICHLET) launch(laplacian_residual_kernel<T, true>);
+    else launch(laplacian_residual_kernel<T, false>);
+    SDFT_CUDA(cudaGetLastError());
+    count_launch(c);
+}
+
+// One FP64 AAR iteration but for the Anderson step, in one launch: r = residual of x, the history push with
+// f = c r (anderson_push_kernel), and either the Richardson step into the other x buffer, xn = omega c r + x, or
+// (xn null, an Anderson step follows) r itself.  Separate kernels for these read x, r and the previous iterate
+// again and cost two more launches per iteration (two-atom cell, 24^3: 4.8 + 1.9 + 1.7 us -> 4.1 us).
+template <bool DIR>
+__global__ void __launch_bounds__(256)
+aar_step_kernel(const double* __restrict__ x, const double* __restrict__ b, double* __restrict__ r_out,
+                double* __restrict__ xn, double* __restrict__ xprev, double* __restrict__ fprev, double* __restrict__ Xs,
+                double* __restrict__ Fs, const __grid_constant__ LapCoef K, int n1, int n2, int n3, double shift,
+                double cj, double wcj, int have_prev) {
+    const int g = blockIdx.x * blockDim.x + threadIdx.x;
+    if (g >= n1 * n2 * n3) return;
+    const double r = laplacian_residual_at<double, DIR>(x, b, K, n1, n2, n3, shift, g);
+    const double xg = x[g];
+    if (have_prev) {
+        Xs[g] = xg - xprev[g];
+        Fs[g] = __dsub_rn(__dmul_rn(cj, r), fprev[g]);
     }
-    K.c0 = c->coef.c0;
-    laplacian_residual_kernel<T><<<(unsigned)((c->ng + 255) / 256), 256, 0, c->stream>>>(
-        x, b, out, K, c->n[0], c->n[1], c->n[2], shift, c->opt.boundary == SDFT_BC_DIRICHLET ? 1 : 0);
+    xprev[g] = xg;
+    fprev[g] = cj * r;
+    if (xn) xn[g] = fma(wcj, r, xg);
+    else r_out[g] = r;
+}
+
+void aar_step(sdft_ctx* c, const double* x, const double* b, double* r, double* xn, double* xprev, double* fprev,
+              double* Xs, double* Fs, double shift, double cj, double omega, bool have_prev) {
+    const LapCoef K = lap_coef<double>(c);
+    // small grids: CTAs small enough that every SM's (few) FP64 pipes get one
+    const int bs = (int)std::min<long long>(256, (c->ng + 152 * 32 - 1) / (152 * 32) * 32);
+    auto launch = [&](auto kfn) {
+        kfn<<<(unsigned)((c->ng + bs - 1) / bs), bs, 0, c->stream>>>(x, b, r, xn, xprev, fprev, Xs, Fs, K, c->n[0],
+                                                                    c->n[1], c->n[2], shift, cj, omega * cj, have_prev);
+    };
+    if (c->opt.boundary == SDFT_BC_DIRICHLET) launch(aar_step_kernel<true>);
+    else launch(aar_step_kernel<false>);
     SDFT_CUDA(cudaGetLastError());
     count_launch(c);
 }
@@ -1089,13 +1245,7 @@ static void isolated_poisson_rhs(sdft_ctx* c, const double* f, double* rhs) {
     double* dq = c->scal + 1700;   // [1700, 1749): multipole moments (free part of the scalar area)
     std::memcpy(c->hscal + 1700, q, sizeof(q));
     SDFT_CUDA(cudaMemcpyAsync(dq, c->hscal + 1700, sizeof(q), cudaMemcpyHostToDevice, c->stream));
-    LapCoef K;
-    for (int r = 0; r <= FD_RADIUS; ++r) {
-        K.c[0][r] = c->coef.cx[r];
-        K.c[1][r] = c->coef.cy[r];
-        K.c[2][r] = c->coef.cz[r];
-    }
-    K.c0 = c->coef.c0;
+    const LapCoef K = lap_coef<double>(c);
     dirichlet_rhs_kernel<<<nblocks(c->ng), 256, 0, c->stream>>>(f, rhs, dq, K, c->n[0], c->n[1], c->n[2], c->h[0],
                                                                c->h[1], c->h[2], cen[0], cen[1], cen[2]);
     SDFT_CUDA(cudaGetLastError());
@@ -1160,47 +1310,42 @@ int poisson_aar(sdft_ctx* c, const double* f, double* phi, double tol, int max_i
     const double cj = 1.0 / (2.0 * c->coef.c0);
     int count = 0, head = 0, it = 0;
     int hslots[16];
-    for (it = 0; it < max_iter; ++it) {
-        // r = rhs - A phi = rhs + L phi  (stencil: alpha=-2 on -1/2 L, beta=-1 on rhs)
-        laplacian_residual<double>(c, phi, rhs, r);
-        // history push with f = cj * r
+    double* buf[2] = {phi, c->work64 + 2 * n};   // the iterate alternates: a Richardson step writes the other buffer
+    int cur = 0;
+    bool done = false;
+    for (it = 0; it < max_iter && !done; ++it) {
+        // r = rhs - A phi = rhs + L phi, history push with f = cj * r, and the Richardson step phi += omega cj r
         const int slot = head;
-        anderson_push_kernel<double><<<nblocks(n), 256, 0, c->stream>>>(phi, r, cj, xprev, fprev, Xs + (long long)slot * n,
-                                                                Fs + (long long)slot * n, it > 0, n);
-        count_launch(c);
         if (it > 0) {
             head = (head + 1) % m;
             count = std::min(count + 1, m);
         }
         const bool anderson = ((it + 1) % p == 0) && count > 0;
-        if (anderson) {
-            for (int j = 0; j < count; ++j) hslots[j] = ((head - count + j) % m + m) % m;
-            std::memcpy(c->hscal + 512, hslots, sizeof(int) * 16);
-            SDFT_CUDA(cudaMemcpyAsync(slots, c->hscal + 512, sizeof(int) * count, cudaMemcpyHostToDevice, c->stream));
-            const int nblk = 64;
-            anderson_gram_kernel<double><<<nblk, RB, 0, c->stream>>>(Fs, slots, count, r, cj, n, part);
-            anderson_solve_kernel<<<1, 256, 0, c->stream>>>(part, nblk, count, gam, ffv);
-            anderson_update_kernel<double><<<nblocks(n), 256, 0, c->stream>>>(phi, r, cj, beta, Xs, Fs, slots, gam, count, n);
-            SDFT_CUDA(cudaGetLastError());
-            count_launch(c, 3);
-            // convergence: ||r||^2 = ffv / cj^2
-            SDFT_CUDA(cudaMemcpyAsync(c->hscal, ffv, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-            SDFT_CUDA(cudaStreamSynchronize(c->stream));
-            const double rn2 = c->hscal[0] / (cj * cj);
-            if (!std::isfinite(rn2)) throw Error{SDFT_ERR_NONFINITE, "Poisson residual is not finite"};
-            if (rn2 <= tol * tol * bnorm2) {
-                ++it;
-                break;
-            }
-        } else {
-            // Richardson: phi += omega * cj * r
-            axpby_kernel<double><<<nblocks(n), 256, 0, c->stream>>>(phi, r, omega * cj, 1.0, n);
-            SDFT_CUDA(cudaGetLastError());
-            count_launch(c);
+        aar_step(c, buf[cur], rhs, r, anderson ? nullptr : buf[cur ^ 1], xprev, fprev, Xs + (long long)slot * n,
+                 Fs + (long long)slot * n, 0.0, cj, omega, it > 0);
+        if (!anderson) {
+            cur ^= 1;
+            continue;
         }
+        for (int j = 0; j < count; ++j) hslots[j] = ((head - count + j) % m + m) % m;
+        std::memcpy(c->hscal + 512, hslots, sizeof(int) * 16);
+        SDFT_CUDA(cudaMemcpyAsync(slots, c->hscal + 512, sizeof(int) * count, cudaMemcpyHostToDevice, c->stream));
+        const int nblk = 64;
+        anderson_gram_kernel<double><<<nblk, RB, 0, c->stream>>>(Fs, slots, count, r, cj, n, part);
+        anderson_solve_kernel<<<1, 256, 0, c->stream>>>(part, nblk, count, gam, ffv);
+        anderson_update_kernel<double><<<nblocks(n), 256, 0, c->stream>>>(buf[cur], r, cj, beta, Xs, Fs, slots, gam,
+                                                                          count, n);
+        SDFT_CUDA(cudaGetLastError());
+        count_launch(c, 3);
+        // convergence: ||r||^2 = ffv / cj^2
+        SDFT_CUDA(cudaMemcpyAsync(c->hscal, ffv, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        SDFT_CUDA(cudaStreamSynchronize(c->stream));
+        const double rn2 = c->hscal[0] / (cj * cj);
+        if (!std::isfinite(rn2)) throw Error{SDFT_ERR_NONFINITE, "Poisson residual is not finite"};
+        done = rn2 <= tol * tol * bnorm2;
     }
-    if (it >= max_iter) return -it;
-    return it;
+    if (cur) SDFT_CUDA(cudaMemcpyAsync(phi, buf[1], sizeof(double) * n, cudaMemcpyDeviceToDevice, c->stream));
+    return it >= max_iter ? -it : it;
 }
 
 // ---------------------------------------------------------------------------------------
@@ -1279,6 +1424,76 @@ static int aar_fp32(sdft_ctx* c, const float* b, float* x, double tol_rel, int m
     return it;
 }
 
+void laplacian_residual_f32(sdft_ctx* c, const float* x, const float* b, float* r) {
+    laplacian_residual<float>(c, x, b, r);
+}
+
+// ---- FP64 passes of the refinement, each with the sum it needs (part[block][k], added by total_kernel) ----
+template <int K>
+__device__ __forceinline__ void block_total(const double (&v)[K], double* __restrict__ part) {
+    __shared__ double sh[K][RB / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        double s = v[k];
+        for (int off = 16; off > 0; off >>= 1) s += __shfl_down_sync(0xffffffffu, s, off);
+        if (lane == 0) sh[k][warp] = s;
+    }
+    __syncthreads();
+    if (threadIdx.x < K) {
+        double s = 0.0;
+        for (int w = 0; w < RB / 32; ++w) s += sh[threadIdx.x][w];
+        part[(long long)blockIdx.x * K + threadIdx.x] = s;
+    }
+}
+// out[k] = sum of part[block][k] over nblk blocks, K <= 2 quantities; one CTA of RB threads
+__global__ void __launch_bounds__(RB) total_kernel(const double* __restrict__ part, int nblk, int K,
+                                                   double* __restrict__ out) {
+    double v[2] = {0.0, 0.0};
+    for (int b = threadIdx.x; b < nblk; b += RB)
+        for (int k = 0; k < K; ++k) v[k] += part[(long long)b * K + k];
+    block_total<2>(v, out);   // two values at out[0], out[1]
+}
+// sums of a and b (b null: of a alone, K = 1 layout)
+__global__ void __launch_bounds__(RB) sum2_kernel(const double* __restrict__ a, const double* __restrict__ b, long long n,
+                                                  double* __restrict__ part) {
+    double v[2] = {0.0, 0.0};
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        v[0] += a[i];
+        if (b) v[1] += b[i];
+    }
+    if (b) block_total<2>(v, part);
+    else block_total<1>({v[0]}, part);
+}
+// rhs = 4 pi (f - mean f), phi -= mean phi (sums = sum f, sum phi), and the sum of rhs^2
+__global__ void __launch_bounds__(RB) poisson_rhs_kernel(const double* __restrict__ f, double* __restrict__ phi,
+                                                         double* __restrict__ rhs, const double* __restrict__ sums,
+                                                         long long n, double* __restrict__ part) {
+    const double mf = sums[0] / (double)n, mp = sums[1] / (double)n;
+    double v[1] = {0.0};
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
+        const double r = 4.0 * M_PI * (f[i] - mf);
+        rhs[i] = r;
+        phi[i] -= mp;
+        v[0] = fma(r, r, v[0]);
+    }
+    block_total<1>(v, part);
+}
+// r = rhs + L phi: its FP32 copy and the sum of r^2
+__global__ void __launch_bounds__(RB) refine_residual_kernel(const double* __restrict__ phi,
+                                                             const double* __restrict__ rhs, float* __restrict__ r32,
+                                                             const __grid_constant__ LapCoef K, int n1, int n2, int n3,
+                                                             double* __restrict__ part) {
+    const int ng = n1 * n2 * n3;
+    double v[1] = {0.0};
+    for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < ng; g += gridDim.x * blockDim.x) {
+        const double r = laplacian_residual_at<double, false>(phi, rhs, K, n1, n2, n3, 0.0, g);
+        r32[g] = (float)r;
+        v[0] = fma(r, r, v[0]);
+    }
+    block_total<1>(v, part);
+}
+
 // FP32 AAR with the multigrid preconditioner M (one V-cycle, poisson_mg.cu) in place of the Jacobi
 // scaling: f_k = M r_k enters the Richardson steps x += omega f and the Anderson extrapolation every
 // p-th step exactly where c r_k does in aar_fp32; convergence is tested on the true residual
@@ -1288,10 +1503,9 @@ static int aar_fp32_mg(sdft_ctx* c, const float* b, float* x, double tol_rel, in
     const long long n = c->ng;
     const float omega = 0.7f, beta = 0.7f;
     const int m = 5, p = 3;
-    // reduction grids: the history Gram's partials (m (m + 1) / 2 + m + 1 = 21 per block) fill 64 * 21
-    // of the 12 288 doubles from scal + 4096, the single dot's 64 of the 1 024 from scal + 2048 (more
-    // blocks did not shorten the Gram, and the one-CTA solve then sums more partials)
-    constexpr int NB_G = 64, NB_R = 64;
+    // reduction grids: the history Gram's partials (m (m + 1) / 2 + m + 1 = 21 per block) fill NB * 21 of the
+    // 12 288 doubles from scal + 4096, the residual's NB of the 1 024 from scal + 2048
+    constexpr int NB = 152;
     float* r = c->work32 + 1 * n;
     float* xprev = c->work32 + 2 * n;
     float* fprev = c->work32 + 3 * n;
@@ -1306,8 +1520,8 @@ static int aar_fp32_mg(sdft_ctx* c, const float* b, float* x, double tol_rel, in
     double* part_r = c->scal + 2048;
     double bnorm2;
     {
-        anderson_gram_kernel<float><<<NB_R, RB, 0, c->stream>>>(Fs, slots, 0, b, 1.0f, n, part_r);
-        anderson_solve_kernel<<<1, 256, 0, c->stream>>>(part_r, NB_R, 0, gam, rrv);
+        anderson_gram_kernel<float><<<NB, RB, 0, c->stream>>>(Fs, slots, 0, b, 1.0f, n, part_r);
+        anderson_solve_kernel<<<1, 256, 0, c->stream>>>(part_r, NB, 0, gam, rrv);
         count_launch(c, 2);
         SDFT_CUDA(cudaMemcpyAsync(c->hscal, rrv, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
         SDFT_CUDA(cudaStreamSynchronize(c->stream));
@@ -1322,41 +1536,31 @@ static int aar_fp32_mg(sdft_ctx* c, const float* b, float* x, double tol_rel, in
     int hslots[16];
     double rel = 1.0;
     for (it = 0; it < max_iter; ++it) {
-        laplacian_residual<float>(c, x, b, r);
-        mg_vcycle(c, r, z);
+        mg_residual_vcycle(c, x, b, r, z);
         const int slot = head;
-        anderson_push_kernel<float><<<nblocks(n), 256, 0, c->stream>>>(x, z, 1.0f, xprev, fprev, Xs + (long long)slot * n,
-                                                                       Fs + (long long)slot * n, it > 0, n);
-        count_launch(c);
         if (it > 0) {
             head = (head + 1) % m;
             count = std::min(count + 1, m);
         }
         const bool anderson = ((it + 1) % p == 0) && count > 0;
-        if (anderson) {
-            for (int j = 0; j < count; ++j) hslots[j] = ((head - count + j) % m + m) % m;
-            std::memcpy(c->hscal + 512, hslots, sizeof(int) * 16);
-            SDFT_CUDA(cudaMemcpyAsync(slots, c->hscal + 512, sizeof(int) * count, cudaMemcpyHostToDevice, c->stream));
-            anderson_gram_kernel<float><<<NB_G, RB, 0, c->stream>>>(Fs, slots, count, z, 1.0f, n, part);
-            anderson_solve_kernel<<<1, 256, 0, c->stream>>>(part, NB_G, count, gam, ffv);
-            // ||r||^2 of the residual this step was taken from
-            anderson_gram_kernel<float><<<NB_R, RB, 0, c->stream>>>(Fs, slots, 0, r, 1.0f, n, part_r);
-            anderson_solve_kernel<<<1, 256, 0, c->stream>>>(part_r, NB_R, 0, gam + 16, rrv);
-            anderson_update_kernel<float><<<nblocks(n), 256, 0, c->stream>>>(x, z, 1.0f, beta, Xs, Fs, slots, gam, count, n);
-            SDFT_CUDA(cudaGetLastError());
-            count_launch(c, 5);
-            SDFT_CUDA(cudaMemcpyAsync(c->hscal, rrv, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-            SDFT_CUDA(cudaStreamSynchronize(c->stream));
-            rel = std::sqrt(c->hscal[0] / bnorm2);
-            if (!std::isfinite(rel)) throw Error{SDFT_ERR_NONFINITE, "Poisson residual is not finite"};
-            if (rel <= tol_rel) {
-                ++it;
-                break;
-            }
-        } else {
-            axpby_kernel<float><<<nblocks(n), 256, 0, c->stream>>>(x, z, omega, 1.0f, n);
-            SDFT_CUDA(cudaGetLastError());
-            count_launch(c);
+        mg_finish(c, r, z, x, xprev, fprev, Xs + (long long)slot * n, Fs + (long long)slot * n, omega, it > 0, !anderson);
+        if (!anderson) continue;
+        for (int j = 0; j < count; ++j) hslots[j] = ((head - count + j) % m + m) % m;
+        std::memcpy(c->hscal + 512, hslots, sizeof(int) * 16);
+        SDFT_CUDA(cudaMemcpyAsync(slots, c->hscal + 512, sizeof(int) * count, cudaMemcpyHostToDevice, c->stream));
+        // the history Gram, and ||r||^2 of the residual this step was taken from
+        anderson_gram2_kernel<float><<<dim3(NB, 2), RB, 0, c->stream>>>(Fs, slots, count, z, r, 1.0f, n, part, part_r);
+        anderson_solve2_kernel<<<2, 256, 0, c->stream>>>(part, part_r, NB, count, gam, ffv, rrv);
+        anderson_update_kernel<float><<<nblocks(n), 256, 0, c->stream>>>(x, z, 1.0f, beta, Xs, Fs, slots, gam, count, n);
+        SDFT_CUDA(cudaGetLastError());
+        count_launch(c, 3);
+        SDFT_CUDA(cudaMemcpyAsync(c->hscal, rrv, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
+        SDFT_CUDA(cudaStreamSynchronize(c->stream));
+        rel = std::sqrt(c->hscal[0] / bnorm2);
+        if (!std::isfinite(rel)) throw Error{SDFT_ERR_NONFINITE, "Poisson residual is not finite"};
+        if (rel <= tol_rel) {
+            ++it;
+            break;
         }
     }
     *final_rel = rel;
@@ -1507,16 +1711,15 @@ __global__ void __launch_bounds__(AAR_BS) aar_persistent_kernel(AarPersistArgs A
             int sl[AAR_M];
             for (int jj = 0; jj < count; ++jj) sl[jj] = ((head - count + jj) % AAR_M + AAR_M) % AAR_M;
             const int nd = count * (count + 1) / 2 + count + 1;
-            double vals[AAR_ND];
+            double* row = A.part + (long long)blockIdx.x * nd;
             switch (count) {
 #define SDFT_AAR_CASE(CC) \
-    case CC: gram_accum<CC, float>(A.Fs, sl, A.r, A.cj, A.n, lo + threadIdx.x, hi, blockDim.x, vals); break;
+    case CC: gram_accum<CC, AAR_BS / 32>(A.Fs, sl, A.r, A.cj, A.n, lo + threadIdx.x, hi, blockDim.x, row, red); break;
                 SDFT_AAR_CASE(1) SDFT_AAR_CASE(2) SDFT_AAR_CASE(3) SDFT_AAR_CASE(4) SDFT_AAR_CASE(5) SDFT_AAR_CASE(6)
                 SDFT_AAR_CASE(7)
 #undef SDFT_AAR_CASE
                 default: break;
             }
-            block_reduce_partials<AAR_BS / 32>(vals, nd, A.part + (long long)blockIdx.x * nd, red);
             if (!grid_barrier(A.bar, A.expected_blocks, A.spin_limit, A.status)) return;
             anderson_solve_block(A.part, gridDim.x, count, gam_s, &ff_s);
             __syncthreads();
@@ -1561,12 +1764,7 @@ static int aar_fp32_persistent(sdft_ctx* c, const float* b, float* x, double tol
     A.bar = reinterpret_cast<unsigned*>(c->scal + 40);
     A.status = reinterpret_cast<int*>(c->scal + 42);
     A.rel_out = c->scal + 44;
-    for (int r = 0; r <= FD_RADIUS; ++r) {
-        A.K.c[0][r] = c->coef.cx[r];
-        A.K.c[1][r] = c->coef.cy[r];
-        A.K.c[2][r] = c->coef.cz[r];
-    }
-    A.K.c0 = c->coef.c0;
+    A.K = lap_coef<double>(c);
     A.n1 = c->n[0];
     A.n2 = c->n[1];
     A.n3 = c->n[2];
@@ -1633,35 +1831,24 @@ int poisson_mixed(sdft_ctx* c, const double* f, double* phi, double tol, int max
     const long long n = c->ng;
     ScopedTimer timer(c, SDFT_K_POISSON);
     double* rhs = c->work64 + 0 * n;
-    double* r = c->work64 + 1 * n;
-    double* ones = c->work64 + 3 * n;
     float* b32 = c->work32;
     float* d32 = c->work32 + 18 * n;
-    // rhs = 4 pi (f - mean f); phi -= mean(phi)
-    SDFT_CUDA(cudaMemsetAsync(ones, 0, sizeof(double) * n, c->stream));
-    c->hscal[0] = 1.0;
-    SDFT_CUDA(cudaMemcpyAsync(c->scal, c->hscal, sizeof(double), cudaMemcpyHostToDevice, c->stream));
-    add_scalar_kernel<<<nblocks(n), 256, 0, c->stream>>>(ones, c->scal, 1.0, n);
-    {
-        const double* A[2] = {f, phi};
-        const double* B[2] = {ones, ones};
-        double s[2];
-        dots_host(c, 2, A, B, n, s);
-        SDFT_CUDA(cudaMemcpyAsync(rhs, f, sizeof(double) * n, cudaMemcpyDeviceToDevice, c->stream));
-        c->hscal[0] = -s[0] / n;
-        c->hscal[1] = -s[1] / n;
-        SDFT_CUDA(cudaMemcpyAsync(c->scal, c->hscal, 2 * sizeof(double), cudaMemcpyHostToDevice, c->stream));
-        add_scalar_kernel<<<nblocks(n), 256, 0, c->stream>>>(rhs, c->scal, 1.0, n);
-        add_scalar_kernel<<<nblocks(n), 256, 0, c->stream>>>(phi, c->scal + 1, 1.0, n);
-        axpby_kernel<double><<<nblocks(n), 256, 0, c->stream>>>(rhs, rhs, 0.0, 4.0 * M_PI, n);
+    double* part = c->scal + 2048;    // partial sums of two quantities, PB blocks
+    double* sums = c->scal + 1536;
+    constexpr int PB = 256;
+    auto host_sums = [&](int k) {
         SDFT_CUDA(cudaGetLastError());
-        count_launch(c, 4);
-    }
-    double bnorm2;
-    {
-        const double* A[1] = {rhs};
-        dots_host(c, 1, A, A, n, &bnorm2);
-    }
+        SDFT_CUDA(cudaMemcpyAsync(c->hscal, sums, sizeof(double) * k, cudaMemcpyDeviceToHost, c->stream));
+        SDFT_CUDA(cudaStreamSynchronize(c->stream));
+    };
+    // sums[0, 1] = sum f, sum phi;  rhs = 4 pi (f - mean f), phi -= mean(phi), with the sum of rhs^2
+    sum2_kernel<<<PB, RB, 0, c->stream>>>(f, phi, n, part);
+    total_kernel<<<1, 256, 0, c->stream>>>(part, PB, 2, sums);
+    poisson_rhs_kernel<<<PB, RB, 0, c->stream>>>(f, phi, rhs, sums, n, part);
+    total_kernel<<<1, 256, 0, c->stream>>>(part, PB, 1, sums);
+    count_launch(c, 4);
+    host_sums(1);
+    const double bnorm2 = c->hscal[0];
     if (bnorm2 == 0.0) {
         SDFT_CUDA(cudaMemsetAsync(phi, 0, sizeof(double) * n, c->stream));
         return 0;
@@ -1669,25 +1856,22 @@ int poisson_mixed(sdft_ctx* c, const double* f, double* phi, double tol, int max
     // zero-mean gauge: FP32 corrections drift along the constant null vector of L, which the
     // residual cannot see, so the mean is removed from phi at the end
     auto remove_mean = [&]() {
-        const double* A[1] = {phi};
-        const double* B[1] = {ones};
-        double sphi;
-        dots_host(c, 1, A, B, n, &sphi);
-        c->hscal[0] = -sphi / n;
-        SDFT_CUDA(cudaMemcpyAsync(c->scal, c->hscal, sizeof(double), cudaMemcpyHostToDevice, c->stream));
-        add_scalar_kernel<<<nblocks(n), 256, 0, c->stream>>>(phi, c->scal, 1.0, n);
-        count_launch(c);
+        sum2_kernel<<<PB, RB, 0, c->stream>>>(phi, nullptr, n, part);
+        total_kernel<<<1, 256, 0, c->stream>>>(part, PB, 1, sums);
+        add_scalar_kernel<<<nblocks(n), 256, 0, c->stream>>>(phi, sums, -1.0 / (double)n, n);
+        SDFT_CUDA(cudaGetLastError());
+        count_launch(c, 3);
     };
+    const LapCoef K = lap_coef<double>(c);
     int total = 0;
     for (int refine = 0; refine < 16; ++refine) {
-        // FP64 residual r = rhs + L phi
-        laplacian_residual<double>(c, phi, rhs, r);
-        double rn2;
-        {
-            const double* A[1] = {r};
-            dots_host(c, 1, A, A, n, &rn2);
-        }
-        const double rel = std::sqrt(rn2 / bnorm2);
+        // FP64 residual r = rhs + L phi: its norm, and its FP32 copy as the next correction's right-hand side
+        refine_residual_kernel<<<(unsigned)std::min<long long>((n + RB - 1) / RB, 1024), RB, 0, c->stream>>>(
+            phi, rhs, b32, K, c->n[0], c->n[1], c->n[2], part);
+        total_kernel<<<1, 256, 0, c->stream>>>(part, (int)std::min<long long>((n + RB - 1) / RB, 1024), 1, sums);
+        count_launch(c, 2);
+        host_sums(1);
+        const double rel = std::sqrt(c->hscal[0] / bnorm2);
         if (!std::isfinite(rel)) throw Error{SDFT_ERR_NONFINITE, "Poisson residual is not finite"};
         if (rel <= tol) {
             remove_mean();
@@ -1696,8 +1880,6 @@ int poisson_mixed(sdft_ctx* c, const double* f, double* phi, double tol, int max
         if (total >= max_iter) break;
         // FP32 correction A d = r: a relative reduction of 1e-3 per refinement stays above the
         // FP32 rounding floor of the residual (~ cond(L) * 2^-24)
-        convert_add_kernel<float, double><<<nblocks(n), 256, 0, c->stream>>>(b32, r, 1.0, 0.0, n);
-        count_launch(c);
         double inner_rel = 1.0;
         const double want = std::max(1e-3, 0.3 * tol / rel);
         const int budget = std::min(400, max_iter - total);

@@ -180,9 +180,9 @@ struct sdft_ctx {
     std::vector<sdft::MgLevel> mg;   // multigrid hierarchy (empty: none)
     double mg_lmin = 0.0, mg_lmax = 0.0;   // spectrum bounds of the coarsest grid's operator
     int mg_coarse_iters = 0;              // Chebyshev iterations on the coarsest grid
-    cudaGraphExec_t mg_graph = nullptr;   // the V-cycle's launches for (mg_graph_r, mg_graph_z)
-    const float* mg_graph_r = nullptr;
-    float* mg_graph_z = nullptr;
+    int mg_tail = 0;                      // first level of the one-CTA end of the hierarchy
+    cudaGraphExec_t mg_graph = nullptr;   // the launches of mg_residual_vcycle for the buffers mg_graph_key
+    const float* mg_graph_key[4] = {nullptr, nullptr, nullptr, nullptr};
     int mg_graph_launches = 0;
     bool test_barrier_extra = false;  // test hook: the persistent barrier waits for one CTA too many
     std::vector<cudaEvent_t> ev_free;
@@ -363,9 +363,12 @@ int poisson_aar(sdft_ctx* c, const double* f, double* phi, double tol, int max_i
 // same problem, FP64 residuals + FP32 AAR corrections; returns inner iterations (negative: failed)
 int poisson_mixed(sdft_ctx* c, const double* f, double* phi, double tol, int max_iter);
 // multigrid preconditioner of the FP32 Poisson corrections (poisson_mg.cu): build the hierarchy
-// (false: the grid does not coarsen far enough), and z = M r by one V-cycle
+// (false: the grid does not coarsen far enough); r = b + L x and z = M r by one V-cycle, in two parts
 bool mg_setup(sdft_ctx* c);
-void mg_vcycle(sdft_ctx* c, const float* r, float* z);
+void mg_residual_vcycle(sdft_ctx* c, const float* x, const float* b, float* r, float* z);
+void mg_finish(sdft_ctx* c, const float* r, float* z, float* x, float* xprev, float* zprev, float* Xs, float* Fs,
+               float omega, bool have_prev, bool richardson);
+void laplacian_residual_f32(sdft_ctx* c, const float* x, const float* b, float* r);
 // reductions: out[i] = sum_g a_i[g] * b_i[g] (device scal), returned synchronously to host
 void dots_host(sdft_ctx* c, int count, const double* const* a, const double* const* b, long long n,
                double* host_out);

@@ -43,104 +43,215 @@ __device__ __forceinline__ float apply_a2(const float* __restrict__ x, const MgD
     return d.diag * xc - (d.w1 * sx + d.w2 * sy + d.w3 * sz);
 }
 
-// red-black Gauss-Seidel half sweep over the points with (i + j + k) & 1 == color (n1, n2, n3 even,
-// so the six neighbours of a point all have the other colour); zero != 0: x is taken as zero
-// (the first half sweep of a cycle, which then needs no cleared buffer)
-__global__ void __launch_bounds__(256) mg_rbgs_kernel(float* __restrict__ x, const float* __restrict__ b, MgDims d,
-                                                      int color, int zero) {
-    const int half = d.n1 >> 1;
-    const int npts = half * d.n2 * d.n3;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < npts; t += gridDim.x * blockDim.x) {
-        const int q = t % half, row = t / half;
-        const int j = row % d.n2, k = row / d.n2;
-        const int i = 2 * q + ((j + k + color) & 1);
-        const int g = row * d.n1 + i;
-        float s = b[g];
-        if (!zero) {
-            const int rowj = row * d.n1;
-            s += d.w1 * (x[rowj + wrapi(i + 1, d.n1)] + x[rowj + wrapi(i - 1, d.n1)]);
-            s += d.w2 * (x[(k * d.n2 + wrapi(j + 1, d.n2)) * d.n1 + i] + x[(k * d.n2 + wrapi(j - 1, d.n2)) * d.n1 + i]);
-            s += d.w3 * (x[(wrapi(k + 1, d.n3) * d.n2 + j) * d.n1 + i] + x[(wrapi(k - 1, d.n3) * d.n2 + j) * d.n1 + i]);
-        }
-        x[g] = s / d.diag;
-    }
+// One red-black sweep before and one after the coarse correction, fused so that a level takes four launches of
+// which each reads what it needs once (the plain form was seven: two half sweeps, restriction of the residual at
+// every point, prolongation, two half sweeps; 20 to 25 launches and 74 us a cycle at 80^3, 53 us now):
+//   * the sweep before starts from zero, so a red point is b / diag and a black one needs b alone: one pass;
+//   * after it the residual of a black point is zero but for rounding, so the restriction visits the 13 red points
+//     of the 27 of a coarse point's stencil (2I, 2J, 2K is red);
+//   * in the sweep after (black, then red) a black point's new value needs the prolonged red neighbours and a red
+//     point's the new black ones: the prolonged values are formed where they are read and never stored.
+// Red points are those with even i + j + k; the levels that are swept have even dimensions, so a point's six
+// neighbours have the other colour.
+struct Pt {
+    int i, j, k;
+};
+__device__ __forceinline__ Pt point_of(int t, int n1, int n2) {
+    const int row = t / n1;
+    Pt p;
+    p.i = t - row * n1;
+    p.k = row / n2;
+    p.j = row - p.k * n2;
+    return p;
+}
+// the six neighbours' values f(i, j, k), weighted by the level's 1 / h^2
+template <typename F>
+__device__ __forceinline__ float neighbours(const MgDims& d, Pt p, F f) {
+    float s = d.w1 * (f(wrapi(p.i + 1, d.n1), p.j, p.k) + f(wrapi(p.i - 1, d.n1), p.j, p.k));
+    s += d.w2 * (f(p.i, wrapi(p.j + 1, d.n2), p.k) + f(p.i, wrapi(p.j - 1, d.n2), p.k));
+    s += d.w3 * (f(p.i, p.j, wrapi(p.k + 1, d.n3)) + f(p.i, p.j, wrapi(p.k - 1, d.n3)));
+    return s;
+}
+__device__ __forceinline__ int at(const MgDims& d, int i, int j, int k) { return (k * d.n2 + j) * d.n1 + i; }
+
+// x after the first sweep at point t
+__device__ __forceinline__ float pre_sweep(const float* __restrict__ b, const MgDims& d, int t, float idiag) {
+    const Pt p = point_of(t, d.n1, d.n2);
+    if (((p.i + p.j + p.k) & 1) == 0) return b[t] * idiag;
+    return (b[t] + idiag * neighbours(d, p, [&](int i, int j, int k) { return b[at(d, i, j, k)]; })) * idiag;
+}
+// full weighting of the residual at coarse point (I, J, K): sum over the fine points (2I + a, 2J + b, 2K + c),
+// a, b, c in {-1, 0, 1}, of w_a w_b w_c (b - A2 x), w_0 = 1/2, w_+-1 = 1/4, red points only
+__device__ __forceinline__ float restrict_red(const float* __restrict__ x, const float* __restrict__ b, const MgDims& f,
+                                              Pt c) {
+    auto res = [&](int a, int bb, int cc) {
+        Pt p{wrapi(2 * c.i + a, f.n1), wrapi(2 * c.j + bb, f.n2), wrapi(2 * c.k + cc, f.n3)};
+        const int g = at(f, p.i, p.j, p.k);
+        return b[g] - (f.diag * x[g] - neighbours(f, p, [&](int i, int j, int k) { return x[at(f, i, j, k)]; }));
+    };
+    float e = 0.f;
+#pragma unroll
+    for (int u = -1; u <= 1; u += 2)
+#pragma unroll
+        for (int v = -1; v <= 1; v += 2) e += res(u, v, 0) + res(u, 0, v) + res(0, u, v);
+    return 0.125f * res(0, 0, 0) + 0.03125f * e;
+}
+// trilinear interpolation of the coarse correction at fine point (i, j, k): fine point 2I + 1 lies between I and I + 1
+__device__ __forceinline__ float prolong(const float* __restrict__ xc, const MgDims& c, int i, int j, int k) {
+    const int i0 = i >> 1, j0 = j >> 1, k0 = k >> 1;
+    const int i1 = (i & 1) ? wrapi(i0 + 1, c.n1) : i0;
+    const int j1 = (j & 1) ? wrapi(j0 + 1, c.n2) : j0;
+    const int k1 = (k & 1) ? wrapi(k0 + 1, c.n3) : k0;
+    return 0.125f * (xc[at(c, i0, j0, k0)] + xc[at(c, i1, j0, k0)] + xc[at(c, i0, j1, k0)] + xc[at(c, i1, j1, k0)] +
+                     xc[at(c, i0, j0, k1)] + xc[at(c, i1, j0, k1)] + xc[at(c, i0, j1, k1)] + xc[at(c, i1, j1, k1)]);
+}
+// point number t of one colour (n1 / 2 per row)
+__device__ __forceinline__ Pt colour_point(int t, const MgDims& d, int colour) {
+    const int half = d.n1 >> 1, row = t / half;
+    Pt p;
+    p.k = row / d.n2;
+    p.j = row - p.k * d.n2;
+    p.i = 2 * (t - row * half) + ((p.j + p.k + colour) & 1);
+    return p;
+}
+__device__ __forceinline__ float post_black(const float* __restrict__ x, const float* __restrict__ b, const MgDims& d,
+                                            const float* __restrict__ xc, const MgDims& c, Pt p, float idiag) {
+    return (b[at(d, p.i, p.j, p.k)] + neighbours(d, p, [&](int i, int j, int k) {
+                return x[at(d, i, j, k)] + prolong(xc, c, i, j, k);
+            })) * idiag;
+}
+__device__ __forceinline__ float post_red(const float* __restrict__ x, const float* __restrict__ b, const MgDims& d,
+                                          Pt p, float idiag) {
+    return (b[at(d, p.i, p.j, p.k)] + neighbours(d, p, [&](int i, int j, int k) { return x[at(d, i, j, k)]; })) * idiag;
 }
 
-// b_c[I, J, K] = sum over the 27 fine points (2I + a, 2J + b, 2K + c), a, b, c in {-1, 0, 1}, of
-// w_a w_b w_c (b_f - A2 x_f), w_0 = 1/2, w_+-1 = 1/4 (full weighting; the weights sum to one)
-__global__ void __launch_bounds__(256) mg_restrict_kernel(const float* __restrict__ xf, const float* __restrict__ bf,
+__global__ void __launch_bounds__(256) mg_pre_kernel(float* __restrict__ x, const float* __restrict__ b, MgDims d) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < d.n1 * d.n2 * d.n3) x[t] = pre_sweep(b, d, t, 1.f / d.diag);
+}
+__global__ void __launch_bounds__(128) mg_restrict_kernel(const float* __restrict__ x, const float* __restrict__ b,
                                                           MgDims f, float* __restrict__ bc, MgDims c) {
-    const int npts = c.n1 * c.n2 * c.n3;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < npts; t += gridDim.x * blockDim.x) {
-        const int I = t % c.n1, row = t / c.n1;
-        const int J = row % c.n2, K = row / c.n2;
-        float acc = 0.f;
-        for (int dk = -1; dk <= 1; ++dk) {
-            const int k = wrapi(2 * K + dk, f.n3);
-            const float wk = dk == 0 ? 0.5f : 0.25f;
-            for (int dj = -1; dj <= 1; ++dj) {
-                const int j = wrapi(2 * J + dj, f.n2);
-                const float wjk = wk * (dj == 0 ? 0.5f : 0.25f);
-                for (int di = -1; di <= 1; ++di) {
-                    const int i = wrapi(2 * I + di, f.n1);
-                    const float r = bf[(k * f.n2 + j) * f.n1 + i] - apply_a2(xf, f, i, j, k);
-                    acc += wjk * (di == 0 ? 0.5f : 0.25f) * r;
-                }
-            }
-        }
-        bc[t] = acc;
-    }
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t < c.n1 * c.n2 * c.n3) bc[t] = restrict_red(x, b, f, point_of(t, c.n1, c.n2));
+}
+__global__ void __launch_bounds__(128) mg_black_kernel(float* __restrict__ x, const float* __restrict__ b, MgDims d,
+                                                       const float* __restrict__ xc, MgDims c) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (d.n1 >> 1) * d.n2 * d.n3) return;
+    const Pt p = colour_point(t, d, 1);
+    // black points are written, red ones read
+    x[at(d, p.i, p.j, p.k)] = post_black(x, b, d, xc, c, p, 1.f / d.diag);
+}
+__global__ void __launch_bounds__(256) mg_red_kernel(float* __restrict__ x, const float* __restrict__ b, MgDims d) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= (d.n1 >> 1) * d.n2 * d.n3) return;
+    const Pt p = colour_point(t, d, 0);
+    x[at(d, p.i, p.j, p.k)] = post_red(x, b, d, p, 1.f / d.diag);
 }
 
-// x_f += P x_c: trilinear interpolation, fine point 2I + 1 between coarse points I and I + 1
-__global__ void __launch_bounds__(256) mg_prolong_kernel(float* __restrict__ xf, MgDims f, const float* __restrict__ xc,
-                                                         MgDims c) {
-    const int npts = f.n1 * f.n2 * f.n3;
-    for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < npts; t += gridDim.x * blockDim.x) {
-        const int i = t % f.n1, row = t / f.n1;
-        const int j = row % f.n2, k = row / f.n2;
-        const int i0 = i >> 1, j0 = j >> 1, k0 = k >> 1;
-        const int i1 = (i & 1) ? wrapi(i0 + 1, c.n1) : i0;
-        const int j1 = (j & 1) ? wrapi(j0 + 1, c.n2) : j0;
-        const int k1 = (k & 1) ? wrapi(k0 + 1, c.n3) : k0;
-        auto at = [&](int a, int b_, int cc) { return xc[(cc * c.n2 + b_) * c.n1 + a]; };
-        const float v = 0.125f * (at(i0, j0, k0) + at(i1, j0, k0) + at(i0, j1, k0) + at(i1, j1, k0) + at(i0, j0, k1) +
-                                  at(i1, j0, k1) + at(i0, j1, k1) + at(i1, j1, k1));
-        xf[t] += v;
+// The finest level's last half sweep together with what the AAR iteration does with z = M r: the history push
+// (X = x - x_prev, F = z - z_prev), and either the Richardson step x += omega z or, when an Anderson step follows, z.
+__global__ void __launch_bounds__(256)
+mg_finish_kernel(float* __restrict__ z, const float* __restrict__ b, MgDims d, float* __restrict__ x,
+                 float* __restrict__ xprev, float* __restrict__ zprev, float* __restrict__ Xs, float* __restrict__ Fs,
+                 float omega, int have_prev, int richardson) {
+    const int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= d.n1 * d.n2 * d.n3) return;
+    const Pt p = point_of(t, d.n1, d.n2);
+    const bool red = ((p.i + p.j + p.k) & 1) == 0;
+    const float zt = red ? post_red(z, b, d, p, 1.f / d.diag) : z[t];   // red points of z are written, black ones read
+    const float xt = x[t];
+    if (have_prev) {
+        Xs[t] = xt - xprev[t];
+        Fs[t] = zt - zprev[t];
     }
+    xprev[t] = xt;
+    zprev[t] = zt;
+    if (richardson) x[t] = xt + omega * zt;
+    else if (red) z[t] = zt;
 }
 
-// coarsest grid: K Chebyshev iterations for A2 x = b from x = 0, for the spectrum [lmin, lmax] of A2
-// without its zero eigenvalue (Saad, Iterative Methods for Sparse Linear Systems, Algorithm 12.1),
-// one CTA, x and the step d in shared memory
-__global__ void __launch_bounds__(1024) mg_coarse_kernel(float* __restrict__ x, const float* __restrict__ b, MgDims d,
-                                                         float lmin, float lmax, int K) {
+// The small end of the hierarchy (levels of up to a few thousand points) in one CTA, all fields in shared memory: a
+// launch per half sweep there costs more than the work.  Levels 0..nl-1 of `A`; the last one is the coarsest grid
+// (nl = 1: the coarsest grid alone), solved by K Chebyshev iterations for A2 x = b from x = 0, for the spectrum
+// [lmin, lmax] of A2 without its zero eigenvalue (Saad, Iterative Methods for Sparse Linear Systems, Algorithm 12.1).
+constexpr int MG_TAIL = 8;
+struct MgTail {
+    MgDims d[MG_TAIL];
+    int off_x[MG_TAIL], off_b[MG_TAIL];   // float offsets into shared memory
+    int nl, off_d;                        // off_d: the Chebyshev step of the coarsest grid
+    float lmin, lmax;
+    int K;
+};
+__global__ void __launch_bounds__(1024) mg_tail_kernel(float* __restrict__ x, const float* __restrict__ b,
+                                                       const __grid_constant__ MgTail A) {
     extern __shared__ float sm[];
-    const int n = d.n1 * d.n2 * d.n3;
-    float* xs = sm;
-    float* ds = sm + n;
-    const float theta = 0.5f * (lmax + lmin), delta = 0.5f * (lmax - lmin);
-    const float sigma1 = theta / delta;
-    for (int p = threadIdx.x; p < n; p += blockDim.x) {
-        ds[p] = b[p] / theta;
-        xs[p] = ds[p];
-    }
-    float rho = 1.f / sigma1;
-    for (int it = 1; it < K; ++it) {
-        __syncthreads();
-        const float rho1 = 1.f / (2.f * sigma1 - rho);
-        for (int p = threadIdx.x; p < n; p += blockDim.x) {
-            const int i = p % d.n1, row = p / d.n1;
-            const int j = row % d.n2, k = row / d.n2;
-            const float r = b[p] - apply_a2(xs, d, i, j, k);
-            ds[p] = rho1 * rho * ds[p] + (2.f * rho1 / delta) * r;
-        }
-        __syncthreads();
-        for (int p = threadIdx.x; p < n; p += blockDim.x) xs[p] += ds[p];
-        rho = rho1;
+    const int nt = blockDim.x, tid = threadIdx.x;
+    {
+        const int n = A.d[0].n1 * A.d[0].n2 * A.d[0].n3;
+        for (int t = tid; t < n; t += nt) sm[A.off_b[0] + t] = b[t];
     }
     __syncthreads();
-    for (int p = threadIdx.x; p < n; p += blockDim.x) x[p] = xs[p];
+    for (int l = 0; l + 1 < A.nl; ++l) {
+        const MgDims& d = A.d[l];
+        const MgDims& c = A.d[l + 1];
+        float* xl = sm + A.off_x[l];
+        const float* bl = sm + A.off_b[l];
+        for (int t = tid; t < d.n1 * d.n2 * d.n3; t += nt) xl[t] = pre_sweep(bl, d, t, 1.f / d.diag);
+        __syncthreads();
+        for (int t = tid; t < c.n1 * c.n2 * c.n3; t += nt)
+            sm[A.off_b[l + 1] + t] = restrict_red(xl, bl, d, point_of(t, c.n1, c.n2));
+        __syncthreads();
+    }
+    {
+        const MgDims& d = A.d[A.nl - 1];
+        const int n = d.n1 * d.n2 * d.n3;
+        float* xs = sm + A.off_x[A.nl - 1];
+        const float* bs = sm + A.off_b[A.nl - 1];
+        float* ds = sm + A.off_d;
+        const float theta = 0.5f * (A.lmax + A.lmin), delta = 0.5f * (A.lmax - A.lmin);
+        const float sigma1 = theta / delta;
+        for (int p = tid; p < n; p += nt) {
+            ds[p] = bs[p] / theta;
+            xs[p] = ds[p];
+        }
+        float rho = 1.f / sigma1;
+        for (int it = 1; it < A.K; ++it) {
+            __syncthreads();
+            const float rho1 = 1.f / (2.f * sigma1 - rho);
+            for (int t = tid; t < n; t += nt) {
+                const Pt p = point_of(t, d.n1, d.n2);
+                const float r = bs[t] - apply_a2(xs, d, p.i, p.j, p.k);
+                ds[t] = rho1 * rho * ds[t] + (2.f * rho1 / delta) * r;
+            }
+            __syncthreads();
+            for (int p = tid; p < n; p += nt) xs[p] += ds[p];
+            rho = rho1;
+        }
+        __syncthreads();
+    }
+    for (int l = A.nl - 2; l >= 0; --l) {
+        const MgDims& d = A.d[l];
+        const MgDims& c = A.d[l + 1];
+        float* xl = sm + A.off_x[l];
+        const float* bl = sm + A.off_b[l];
+        const float* xc = sm + A.off_x[l + 1];
+        const int half = (d.n1 >> 1) * d.n2 * d.n3;
+        for (int t = tid; t < half; t += nt) {
+            const Pt p = colour_point(t, d, 1);
+            xl[at(d, p.i, p.j, p.k)] = post_black(xl, bl, d, xc, c, p, 1.f / d.diag);
+        }
+        __syncthreads();
+        for (int t = tid; t < half; t += nt) {
+            const Pt p = colour_point(t, d, 0);
+            xl[at(d, p.i, p.j, p.k)] = post_red(xl, bl, d, p, 1.f / d.diag);
+        }
+        __syncthreads();
+    }
+    {
+        const int n = A.d[0].n1 * A.d[0].n2 * A.d[0].n3;
+        for (int t = tid; t < n; t += nt) x[t] = sm[A.off_x[0] + t];
+    }
 }
 
 MgDims dims_of(const MgLevel& L) {
@@ -155,11 +266,13 @@ MgDims dims_of(const MgLevel& L) {
     return d;
 }
 
-unsigned mg_blocks(long long work) { return (unsigned)std::max<long long>(1, std::min<long long>((work + 255) / 256, 152LL * 8)); }
+unsigned mg_blocks(long long work, int bs) { return (unsigned)((work + bs - 1) / bs); }
 
 constexpr int MG_COARSE_STOP = 512;    // coarsening stops once a grid has at most this many points
 constexpr int MG_COARSE_MAX = 16384;   // largest coarsest grid (x and d in shared memory)
-constexpr int MG_NU = 1;               // red-black sweeps before and after the coarse correction
+constexpr size_t MG_TAIL_SMEM = 200 * 1024;   // shared memory of the one-CTA end of the hierarchy
+// its largest swept level: a tail that takes in a 20^3 level costs 34 us; this one 8.6, plus four launches of 2 to 4 us
+constexpr long long MG_TAIL_POINTS = 2048;
 
 }  // namespace
 
@@ -215,74 +328,81 @@ bool mg_setup(sdft_ctx* c) {
     // AAR iteration count in a model of the solver)
     const double sk = std::sqrt(lmax / lmin), q = (sk - 1.0) / (sk + 1.0);
     c->mg_coarse_iters = q <= 0.0 ? 1 : std::min(64, std::max(2, (int)std::ceil(std::log(5e-2) / std::log(q))));
-    // the attribute belongs to the kernel, not to this context: allow the largest coarsest grid of any
-    // context, so that a context created later with a smaller one does not lower it for this one
-    SDFT_CUDA(cudaFuncSetAttribute(mg_coarse_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   (int)(sizeof(float) * 2 * MG_COARSE_MAX)));
+    // levels from mg_tail on run in one CTA: x and b of each (x, b and the step of the coarsest) in shared memory
+    int first = (int)lv.size() - 1;
+    size_t smem = sizeof(float) * 3 * (size_t)cl.np;
+    while (first > 1 && (int)lv.size() - first < MG_TAIL && lv[first - 1].np <= MG_TAIL_POINTS &&
+           smem + sizeof(float) * 2 * (size_t)lv[first - 1].np <= MG_TAIL_SMEM) {
+        --first;
+        smem += sizeof(float) * 2 * (size_t)lv[first].np;
+    }
+    c->mg_tail = first;
+    // the attribute belongs to the kernel, not to this context: allow what any context's tail may need
+    SDFT_CUDA(cudaFuncSetAttribute(mg_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MG_TAIL_SMEM));
     c->mg = lv;
     return true;
 }
 
 namespace {
-// the V-cycle's launches (level 0 uses r and z in place of its own b and x)
+// the launches of z = M r but for the finest level's last half sweep (mg_finish does it): level 0 uses r and z in
+// place of its own b and x
 void mg_enqueue(sdft_ctx* c, const float* r, float* z) {
-    const int nl = (int)c->mg.size();
-    SDFT_REQUIRE(nl >= 2, SDFT_ERR_INVALID_ARG, "multigrid V-cycle without a hierarchy");
-    auto xb = [&](int l, float** x, const float** b) {
-        *x = l == 0 ? z : c->mg[l].x;
-        *b = l == 0 ? r : c->mg[l].b;
-    };
-    for (int l = 0; l + 1 < nl; ++l) {
-        float* x;
-        const float* b;
-        xb(l, &x, &b);
+    const int nl = (int)c->mg.size(), tail = c->mg_tail;
+    SDFT_REQUIRE(nl >= 2 && tail >= 1, SDFT_ERR_INVALID_ARG, "multigrid V-cycle without a hierarchy");
+    auto x = [&](int l) { return l == 0 ? z : c->mg[l].x; };
+    auto b = [&](int l) { return l == 0 ? r : (const float*)c->mg[l].b; };
+    for (int l = 0; l < tail; ++l) {
         const MgDims d = dims_of(c->mg[l]);
-        const unsigned nbh = mg_blocks(c->mg[l].np / 2);
-        for (int s = 0; s < MG_NU; ++s) {
-            mg_rbgs_kernel<<<nbh, 256, 0, c->stream>>>(x, b, d, 0, s == 0 ? 1 : 0);
-            mg_rbgs_kernel<<<nbh, 256, 0, c->stream>>>(x, b, d, 1, 0);
-        }
-        mg_restrict_kernel<<<mg_blocks(c->mg[l + 1].np), 256, 0, c->stream>>>(x, b, d, c->mg[l + 1].b,
-                                                                                 dims_of(c->mg[l + 1]));
-        count_launch(c, 2 * MG_NU + 1);
+        mg_pre_kernel<<<mg_blocks(c->mg[l].np, 256), 256, 0, c->stream>>>(x(l), b(l), d);
+        mg_restrict_kernel<<<mg_blocks(c->mg[l + 1].np, 128), 128, 0, c->stream>>>(x(l), b(l), d, c->mg[l + 1].b,
+                                                                                  dims_of(c->mg[l + 1]));
+        count_launch(c, 2);
     }
     {
-        const MgLevel& cl = c->mg[nl - 1];
-        const size_t smem = sizeof(float) * 2 * (size_t)cl.np;
-        mg_coarse_kernel<<<1, 1024, smem, c->stream>>>(cl.x, cl.b, dims_of(cl), (float)c->mg_lmin, (float)c->mg_lmax,
-                                                        c->mg_coarse_iters);
+        MgTail A{};
+        int off = 0;
+        A.nl = nl - tail;
+        for (int l = 0; l < A.nl; ++l) {
+            const MgLevel& L = c->mg[tail + l];
+            A.d[l] = dims_of(L);
+            A.off_x[l] = off;
+            A.off_b[l] = off + (int)L.np;
+            off += 2 * (int)L.np;
+        }
+        A.off_d = off;
+        off += (int)c->mg[nl - 1].np;
+        A.lmin = (float)c->mg_lmin;
+        A.lmax = (float)c->mg_lmax;
+        A.K = c->mg_coarse_iters;
+        mg_tail_kernel<<<1, 1024, sizeof(float) * (size_t)off, c->stream>>>(c->mg[tail].x, c->mg[tail].b, A);
         count_launch(c);
     }
-    for (int l = nl - 2; l >= 0; --l) {
-        float* x;
-        const float* b;
-        xb(l, &x, &b);
+    for (int l = tail - 1; l >= 0; --l) {
         const MgDims d = dims_of(c->mg[l]);
-        mg_prolong_kernel<<<mg_blocks(c->mg[l].np), 256, 0, c->stream>>>(x, d, c->mg[l + 1].x, dims_of(c->mg[l + 1]));
-        const unsigned nbh = mg_blocks(c->mg[l].np / 2);
-        for (int s = 0; s < MG_NU; ++s) {
-            mg_rbgs_kernel<<<nbh, 256, 0, c->stream>>>(x, b, d, 1, 0);
-            mg_rbgs_kernel<<<nbh, 256, 0, c->stream>>>(x, b, d, 0, 0);
-        }
-        count_launch(c, 2 * MG_NU + 1);
+        mg_black_kernel<<<mg_blocks(c->mg[l].np / 2, 128), 128, 0, c->stream>>>(x(l), b(l), d, c->mg[l + 1].x,
+                                                                               dims_of(c->mg[l + 1]));
+        if (l > 0) mg_red_kernel<<<mg_blocks(c->mg[l].np / 2, 256), 256, 0, c->stream>>>(x(l), b(l), d);
+        count_launch(c, l > 0 ? 2 : 1);
     }
     SDFT_CUDA(cudaGetLastError());
 }
 }  // namespace
 
-// z = M r: one V-cycle from a zero start.  The V-cycle is some twenty small launches, most of them on
-// grids of a few thousand points, so it is captured once into a CUDA graph (for the context's r and
-// z buffers) and replayed; SDFT_MG_GRAPH=0 launches the kernels one by one.
-void mg_vcycle(sdft_ctx* c, const float* r, float* z) {
+// r = b + L x and z = M r (but for the last half sweep, see mg_finish) from a zero start.  About ten small launches
+// with fixed buffers, so they are captured once into a CUDA graph and replayed; SDFT_MG_GRAPH=0 launches them one by
+// one.
+void mg_residual_vcycle(sdft_ctx* c, const float* x, const float* b, float* r, float* z) {
     static const bool use_graph = [] {
         const char* env = getenv("SDFT_MG_GRAPH");
         return env == nullptr || atoi(env) != 0;
     }();
     if (!use_graph) {
+        laplacian_residual_f32(c, x, b, r);
         mg_enqueue(c, r, z);
         return;
     }
-    if (c->mg_graph && (c->mg_graph_r != r || c->mg_graph_z != z)) {
+    const float* key[4] = {x, b, r, z};
+    if (c->mg_graph && !std::equal(key, key + 4, c->mg_graph_key)) {
         cudaGraphExecDestroy(c->mg_graph);
         c->mg_graph = nullptr;
     }
@@ -295,6 +415,7 @@ void mg_vcycle(sdft_ctx* c, const float* r, float* z) {
         c->stream = c->cap_stream;
         SDFT_CUDA(cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal));
         try {
+            laplacian_residual_f32(c, x, b, r);
             mg_enqueue(c, r, z);
         } catch (...) {
             cudaStreamEndCapture(c->stream, &graph);
@@ -310,11 +431,19 @@ void mg_vcycle(sdft_ctx* c, const float* r, float* z) {
         SDFT_CUDA(ie);
         c->mg_graph_launches = (int)(c->launches - l0);
         c->launches = l0;
-        c->mg_graph_r = r;
-        c->mg_graph_z = z;
+        std::copy(key, key + 4, c->mg_graph_key);
     }
     SDFT_CUDA(cudaGraphLaunch(c->mg_graph, c->stream));
     count_launch(c, c->mg_graph_launches);
+}
+
+// the last half sweep of z = M r, the history push and (richardson) the step x += omega z
+void mg_finish(sdft_ctx* c, const float* r, float* z, float* x, float* xprev, float* zprev, float* Xs, float* Fs,
+               float omega, bool have_prev, bool richardson) {
+    mg_finish_kernel<<<mg_blocks(c->ng, 256), 256, 0, c->stream>>>(z, r, dims_of(c->mg[0]), x, xprev, zprev, Xs, Fs,
+                                                                  omega, have_prev, richardson);
+    SDFT_CUDA(cudaGetLastError());
+    count_launch(c);
 }
 
 }  // namespace sdft
