@@ -151,7 +151,7 @@ void build_context(sdft_ctx* c) {
     c->rho_out = (double*)ctx_alloc(c, sizeof(double) * o.nspin * ng);
     c->phi = (double*)ctx_alloc(c, sizeof(double) * ng);
     c->veff = (double*)ctx_alloc(c, sizeof(double) * o.nspin * ng);
-    c->veff32 = (float*)ctx_alloc(c, sizeof(float) * o.nspin * ng);
+    c->veff32 = (float*)ctx_alloc(c, sizeof(float) * (o.nspin * ng + 4));   // + 4: copies in whole 16 bytes
     c->exc = (double*)ctx_alloc(c, sizeof(double) * ng);
     c->work64 = (double*)ctx_alloc(c, sizeof(double) * 28 * ng);
     c->work32 = (float*)ctx_alloc(c, sizeof(float) * 20 * ng);

@@ -336,6 +336,10 @@ template <int N1, int TY, int NP, int RY, int S, int D, int MINB>
 void launch_slab_variant(sdft_ctx* c, int kpt, const float2* Y, const float2* Yprev, float2* Ynext, int ncolE,
                          const float* V, const float2* kbC, double alpha, double beta, double shift, bool kin,
                          bool timed);
+// ---- stencil_slabx.cu: the same for any even n1 --------------------------------------------
+bool slabx_ok(const sdft_ctx* c, int ncolE);
+void launch_slabx(sdft_ctx* c, int kpt, const float2* Y, const float2* Yprev, float2* Ynext, int ncolE, const float* V,
+                  const float2* kbC, double alpha, double beta, double shift, bool kin, bool timed);
 // sticky device flag (int) set by a stencil launch whose bounded mbarrier wait gave up
 int* stencil_error_flag(sdft_ctx* c);
 // throws SDFT_ERR_DEVICE_TIMEOUT if that flag is set (reads it after the stream's work so far)

@@ -278,10 +278,10 @@ void build_kb_tables(sdft_ctx* c, int kpt) {
     T.S = S;
     if (S > 0) {
         const size_t ps = (size_t)S * c->ng;
-        T.patom = (int*)ctx_alloc(c, sizeof(int) * ps);
+        T.patom = (int*)ctx_alloc(c, sizeof(int) * (ps + 4));   // + 4: copies in whole 16 bytes
         SDFT_CUDA(cudaMemsetAsync(T.patom, 0xff, sizeof(int) * ps, c->stream));  // unused slots: atom -1
         T.pval64 = (double*)ctx_alloc(c, sizeof(double) * ps * vw);
-        T.pval32 = (float*)ctx_alloc(c, sizeof(float) * ps * vw);
+        T.pval32 = (float*)ctx_alloc(c, sizeof(float) * (ps * vw + 4));
         int* pfill = (int*)ctx_alloc(c, sizeof(int) * c->ng);
         SDFT_CUDA(cudaMemsetAsync(pfill, 0, sizeof(int) * c->ng, c->stream));
         point_fill_kernel<<<dim3(c->natom, 8), 256, 0, c->stream>>>(T.cnt, T.idx, T.val64, T.val32, T.cap, T.cplx, c->ng, S,

@@ -60,7 +60,8 @@ __device__ __forceinline__ float bf16r(float x) { return __bfloat162float(__floa
 // the same order as a plain loop over the inputs.  Activations are written twice where a product needs them along
 // points (next layer) and along neurons (gradient).  Weight gradients stay in registers over all tiles of the CTA.
 // The kernel this replaces read two scalars from shared memory for every multiply-add of a gradient and kept the
-// gradient there too: 65 536 points, loss and gradient: 255 -> 81 us.
+// gradient there too: 65 536 points, loss and gradient: 255 -> 81 us;
+// 512 000 points, inference: 443 -> 190 us.
 constexpr int MT = 256;              // threads
 constexpr int XS = NF + 4, HS = NH + 4;   // row strides of the point-major copies (conflict-free vector stores)
 struct MlpSmem {

@@ -34,6 +34,7 @@ const StepVariant<float2> kReal[] = {
     // bricks of 8 and 4 planes (stencil_brick.cuh)
     {&launch_brick<float2, false, 8, 2>, &brick_ok<float2, 8>, "brick8"},
     {&launch_brick<float2, false, 4, 2>, &brick_ok<float2, 4>, "brick4"},
+    {&launch_slabx, &slabx_ok, "slabx"},
 };
 const StepVariant<float2> kCplx[] = {
     {&launch_variant<float2, true, 32, 8, 2, 2, 4>, nullptr, "col32x8"},
@@ -45,12 +46,22 @@ const StepVariant<float2> kCplx[] = {
     {&launch_brick<float2, true, 4, 2>, &brick_ok<float2, 4>, "brick4"},
 };
 constexpr int kRealBrick8 = 16, kCplxBrick8 = 5;   // the brick4 variants follow
+constexpr int kRealSlabx = 18;
+constexpr unsigned long long kSlabs = 0x1fULL << 11 | 1ULL << kRealSlabx;   // the TMA-fed slab tiles of kReal
 constexpr int kNReal = sizeof(kReal) / sizeof(kReal[0]);
 constexpr int kNCplx = sizeof(kCplx) / sizeof(kCplx[0]);
 }  // namespace
 
+// Real blocks with rows of 44 points and more (even): only the slab tiles are timed.  us a step, slab and best column, row
+// or brick tile: 80^3, 180 columns 294 and 668; 82 x 82 x 76, 176 columns 358 and 706; 96^3, 300 columns 915 and 1600;
+// 64 x 60 x 60, 66 columns 63 and 115; 48^3, 32 columns 23 and 27.  Shorter rows: 40^3 20.7 and 21.9, 36^3 19.0 and
+// 18.9, 20^3 27 and 18.
+static bool long_rows(const sdft_ctx* c, bool cplx, int ncolE) { return !cplx && c->n[0] >= 44 && slabx_ok(c, ncolE); }
+
 // Calls too small to be timed take a brick tile: 37 x 41 x 45 points, 20 columns: 15.4 us a step, 31 with the column
 // tile; 40^3, 28 columns: 20 and 26; 48^3, 40 columns: 35 and 66.  Bricks of 8 planes need two CTAs an SM, else 4.
+// (The slab would take 29 us for the last of these, but the multi-cell filter runs bricks, and a cell gets the same bits
+// from it as from its own filter.)
 static int small_variant(const sdft_ctx* c, bool cplx, int ncolE) {
     const int v8 = cplx ? kCplxBrick8 : kRealBrick8;
     if (!brick_ok<float2, 8>(c, ncolE)) return 0;
@@ -84,7 +95,8 @@ void launch_cheb_step<float2>(sdft_ctx* c, int kpt, const float2* Y, const float
         c->kb_next = nullptr;
         bool fused = true;
         pick = autotune_stencil<float2>(c, table, nvar, kpt, Y, Yprev, Ynext, ncolE, V, kbC, alpha, beta, shift,
-                                        kb_next, kb_next ? &launch_kb_project<float2> : nullptr, &fused);
+                                        kb_next, kb_next ? &launch_kb_project<float2> : nullptr, &fused,
+                                        long_rows(c, cplx, ncolE) ? kSlabs : ~0ULL);
         c->kb_next = kb_next;
         if (pick >= 0) {   // small calls are not timed and do not fix the choice
             choice = pick;

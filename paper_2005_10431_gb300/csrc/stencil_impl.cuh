@@ -957,7 +957,8 @@ template <typename E>
 int autotune_stencil(sdft_ctx* c, const StepVariant<E>* table, int nvar, int kpt, const E* Y, const E* Yprev,
                      E* Ynext, int ncolE, const typename Elem<E>::S* V, const E* kbC, double alpha, double beta,
                      double shift, E* proj = nullptr,
-                     void (*project)(sdft_ctx*, int, const E*, E*, int) = nullptr, bool* fused = nullptr) {
+                     void (*project)(sdft_ctx*, int, const E*, E*, int) = nullptr, bool* fused = nullptr,
+                     unsigned long long candidates = ~0ULL) {
     auto usable = [&](int v) { return table[v].ok == nullptr || table[v].ok(c, ncolE); };
     if (const char* env = getenv("SDFT_STENCIL_VARIANT")) {
         const int v = atoi(env);
@@ -987,16 +988,20 @@ int autotune_stencil(sdft_ctx* c, const StepVariant<E>* table, int nvar, int kpt
     };
     bool best_fused = false;
     for (int v = 0; v < nvar; ++v) {
-        if (!usable(v)) continue;
+        if (!(candidates >> v & 1) || !usable(v)) continue;
         for (int fuse = 0; fuse < (proj != nullptr ? 2 : 1); ++fuse) {
             const bool f = run(v, fuse != 0);   // warm-up
             if (fuse && !f) break;              // no fused projection in this variant
-            SDFT_CUDA(cudaEventRecord(a, c->stream));
-            for (int r = 0; r < 3; ++r) run(v, fuse != 0);
-            SDFT_CUDA(cudaEventRecord(b, c->stream));
-            SDFT_CUDA(cudaEventSynchronize(b));
             float ms = 0.f;
-            SDFT_CUDA(cudaEventElapsedTime(&ms, a, b));
+            for (int r = 1; r <= 2; ++r) {      // one run, then two more unless it was far from the best
+                SDFT_CUDA(cudaEventRecord(a, c->stream));
+                for (int q = 0; q < r; ++q) run(v, fuse != 0);
+                SDFT_CUDA(cudaEventRecord(b, c->stream));
+                SDFT_CUDA(cudaEventSynchronize(b));
+                SDFT_CUDA(cudaEventElapsedTime(&ms, a, b));
+                ms /= (float)r;
+                if (ms > 1.25f * best_ms) break;
+            }
             if (ms < best_ms) {
                 best_ms = ms;
                 best = v;

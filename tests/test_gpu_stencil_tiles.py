@@ -14,6 +14,7 @@ import workloads  # noqa: E402
 from oracle import chefsi, ham, model  # noqa: E402
 
 BRICK8, BRICK4 = (16, "brick8"), (17, "brick4")
+SLABX = (18, "slabx")
 CBRICK8, CBRICK4 = (5, "brick8"), (6, "brick4")
 
 
@@ -63,6 +64,14 @@ def _check(sd, cell, precision, ns, variant, kred, degree, monkeypatch):
 @pytest.mark.parametrize("variant", [BRICK8, BRICK4])
 def test_brick_tile_matches_oracle(sd, n, ns, natom, variant, monkeypatch):
     _check(sd, _cell(n, natom), sd.SDFT_MIXED, ns, variant, (0.0, 0.0, 0.0), 3, monkeypatch)
+
+
+# rows in one slab and in several, a ragged last slab of one row, halos that wrap more than once, an odd number of
+# points per plane pair (copies that start between 16-byte boundaries), more KB slots than are staged, odd numbers of pairs
+@pytest.mark.parametrize("n,ns,natom", [((14, 7, 6), 2, 1), ((14, 9, 15), 6, 7), ((82, 15, 9), 4, 4), ((46, 27, 13), 10, 2),
+                                        ((160, 9, 7), 6, 3), ((22, 30, 40), 14, 5)])
+def test_slab_of_any_even_row_matches_oracle(sd, n, ns, natom, monkeypatch):
+    _check(sd, _cell(n, natom), sd.SDFT_MIXED, ns, SLABX, (0.0, 0.0, 0.0), 3, monkeypatch)
 
 
 @pytest.mark.parametrize("n,ns,natom", [((6, 7, 6), 2, 1), ((23, 12, 9), 3, 4), ((7, 37, 13), 5, 2)])
