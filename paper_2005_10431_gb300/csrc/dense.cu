@@ -73,7 +73,11 @@ gram_kernel(const void* __restrict__ Y, const void* __restrict__ HY, int ncol, l
     __shared__ A Ar[KS][GT + 1], Ai[C ? KS : 1][GT + 1], Br[KS][GT + 1], Bi[C ? KS : 1][GT + 1], Hr[KS][GT + 1],
         Hi[C ? KS : 1][GT + 1];
     const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    // each thread: outputs (i0 + ty + 16a, j0 + tx + 16b), a, b in {0,1}
+    // each thread: outputs (i0 + ty + 16a, j0 + tx + 16b), a, b in {0,1}; a < na and b < nb where a warp has any such row
+    // and the tile any such column (the multiply-adds of the others were what bound small blocks: 8 FP64 columns of 24^3
+    // points 50 -> 8.6 us)
+    const int row0 = i0 + (ty & ~1);
+    const int na = row0 >= ncol ? 0 : row0 + 16 >= ncol ? 1 : 2, nb = j0 + 16 >= ncol ? 1 : 2;
     A mr[2][2] = {{0, 0}, {0, 0}}, mi[2][2] = {{0, 0}, {0, 0}};
     A hr[2][2] = {{0, 0}, {0, 0}}, hi[2][2] = {{0, 0}, {0, 0}};
     for (long long gb = g0; gb < g1; gb += KS) {
@@ -100,36 +104,47 @@ gram_kernel(const void* __restrict__ Y, const void* __restrict__ HY, int ncol, l
             }
         }
         __syncthreads();
+        auto products = [&](auto na_, auto nb_) {
+            constexpr int NA = decltype(na_)::value, NB = decltype(nb_)::value;
 #pragma unroll 8
-        for (int k = 0; k < KS; ++k) {
-            A ar[2], ai[2], br[2], bi[2], h_r[2], h_i[2];
-            for (int a = 0; a < 2; ++a) {
-                ar[a] = Ar[k][ty + 16 * a];
-                ai[a] = A(0);
-                if constexpr (C) ai[a] = Ai[k][ty + 16 * a];
-            }
-            for (int b = 0; b < 2; ++b) {
-                br[b] = Br[k][tx + 16 * b];
-                h_r[b] = Hr[k][tx + 16 * b];
-                bi[b] = h_i[b] = A(0);
-                if constexpr (C) {
-                    bi[b] = Bi[k][tx + 16 * b];
-                    h_i[b] = Hi[k][tx + 16 * b];
+            for (int k = 0; k < KS; ++k) {
+                A ar[2], ai[2], br[2], bi[2], h_r[2], h_i[2];
+#pragma unroll
+                for (int a = 0; a < NA; ++a) {
+                    ar[a] = Ar[k][ty + 16 * a];
+                    ai[a] = A(0);
+                    if constexpr (C) ai[a] = Ai[k][ty + 16 * a];
                 }
-            }
-            for (int a = 0; a < 2; ++a)
-                for (int b = 0; b < 2; ++b) {
-                    // conj(a) * b
-                    mr[a][b] = fma(ar[a], br[b], mr[a][b]);
-                    hr[a][b] = fma(ar[a], h_r[b], hr[a][b]);
-                    if (C) {
-                        mr[a][b] = fma(ai[a], bi[b], mr[a][b]);
-                        mi[a][b] = fma(ar[a], bi[b], fma(-ai[a], br[b], mi[a][b]));
-                        hr[a][b] = fma(ai[a], h_i[b], hr[a][b]);
-                        hi[a][b] = fma(ar[a], h_i[b], fma(-ai[a], h_r[b], hi[a][b]));
+#pragma unroll
+                for (int b = 0; b < NB; ++b) {
+                    br[b] = Br[k][tx + 16 * b];
+                    h_r[b] = Hr[k][tx + 16 * b];
+                    bi[b] = h_i[b] = A(0);
+                    if constexpr (C) {
+                        bi[b] = Bi[k][tx + 16 * b];
+                        h_i[b] = Hi[k][tx + 16 * b];
                     }
                 }
-        }
+#pragma unroll
+                for (int a = 0; a < NA; ++a)
+#pragma unroll
+                    for (int b = 0; b < NB; ++b) {
+                        // conj(a) * b
+                        mr[a][b] = fma(ar[a], br[b], mr[a][b]);
+                        hr[a][b] = fma(ar[a], h_r[b], hr[a][b]);
+                        if (C) {
+                            mr[a][b] = fma(ai[a], bi[b], mr[a][b]);
+                            mi[a][b] = fma(ar[a], bi[b], fma(-ai[a], br[b], mi[a][b]));
+                            hr[a][b] = fma(ai[a], h_i[b], hr[a][b]);
+                            hi[a][b] = fma(ar[a], h_i[b], fma(-ai[a], h_r[b], hi[a][b]));
+                        }
+                    }
+            }
+        };
+        using One = std::integral_constant<int, 1>;
+        using Two = std::integral_constant<int, 2>;
+        if (na == 2) nb == 2 ? products(Two{}, Two{}) : products(Two{}, One{});
+        else if (na == 1) nb == 2 ? products(One{}, Two{}) : products(One{}, One{});
         __syncthreads();
     }
     const long long nn = (long long)ncol * ncol;
