@@ -280,7 +280,8 @@ __global__ void unscale_rows_kernel(double* __restrict__ Q, const double* __rest
     }
 }
 
-// X = Y Q: tile 64 grid points x 32 columns, k in steps of 32
+// X = Y Q: tile 64 grid points x 32 columns, k in steps of 32.  Terms k and column octets (a warp's) past the block are
+// skipped: a block of 8 FP64 columns did 16 times the multiply-adds it needs (24^3 points: 34 -> 4.5 us).
 template <int KIND>
 __global__ void __launch_bounds__(256)
 rotate_kernel(const void* __restrict__ Y, const void* __restrict__ Q, void* __restrict__ X, int ncol, long long ng) {
@@ -297,17 +298,18 @@ rotate_kernel(const void* __restrict__ Y, const void* __restrict__ Q, void* __re
     for (int j = 0; j < 8; ++j) accr[j] = acci[j] = 0;
     const A* Qa = (const A*)Q;
     for (int k0 = 0; k0 < ncol; k0 += TK) {
-        for (int e = threadIdx.x; e < TG * TK; e += 256) {
+        const int kn = min(TK, ncol - k0);
+        for (int e = threadIdx.x; e < TG * kn; e += 256) {
             const int gg = e % TG, kk = e / TG;
             A re = 0, im = 0;
-            if (g0 + gg < ng && k0 + kk < ncol) ld<KIND>(Y, g0 + gg, k0 + kk, ng, re, im);
+            if (g0 + gg < ng) ld<KIND>(Y, g0 + gg, k0 + kk, ng, re, im);
             Yr[gg][kk] = re;
             if constexpr (C) Yi[gg][kk] = im;
         }
-        for (int e = threadIdx.x; e < TK * TN; e += 256) {
+        for (int e = threadIdx.x; e < kn * TN; e += 256) {
             const int nn = e % TN, kk = e / TN;
             A re = 0, im = 0;
-            if (k0 + kk < ncol && n0 + nn < ncol) {
+            if (n0 + nn < ncol) {
                 const long long o = (long long)(k0 + kk) + (long long)(n0 + nn) * ncol;
                 if (C) {
                     re = Qa[2 * o];
@@ -320,19 +322,21 @@ rotate_kernel(const void* __restrict__ Y, const void* __restrict__ Q, void* __re
             if constexpr (C) Qi[kk][nn] = im;
         }
         __syncthreads();
+        if (n0 + nl < ncol) {
 #pragma unroll 4
-        for (int k = 0; k < TK; ++k) {
-            const A yr = Yr[gl][k];
-            A yi = A(0);
-            if constexpr (C) yi = Yi[gl][k];
+            for (int k = 0; k < kn; ++k) {
+                const A yr = Yr[gl][k];
+                A yi = A(0);
+                if constexpr (C) yi = Yi[gl][k];
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {
-                const A qr = Qr[k][nl + j];
-                accr[j] = fma(yr, qr, accr[j]);
-                if constexpr (C) {
-                    const A qi = Qi[k][nl + j];
-                    accr[j] = fma(-yi, qi, accr[j]);
-                    acci[j] = fma(yr, qi, fma(yi, qr, acci[j]));
+                for (int j = 0; j < 8; ++j) {
+                    const A qr = Qr[k][nl + j];
+                    accr[j] = fma(yr, qr, accr[j]);
+                    if constexpr (C) {
+                        const A qi = Qi[k][nl + j];
+                        accr[j] = fma(-yi, qi, accr[j]);
+                        acci[j] = fma(yr, qi, fma(yi, qr, acci[j]));
+                    }
                 }
             }
         }
