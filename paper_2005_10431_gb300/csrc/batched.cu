@@ -6,7 +6,7 @@
 //   2. Cholesky M' = L L^H
 //   3. A = L^-1 H' L^-H (two triangular solves, then symmetrised)
 //   4. cyclic Jacobi on A with the round-robin (tournament) order: n/2 disjoint rotations per
-//      round, applied as one column pass and one row pass; sweeps until no rotation is needed
+//      round, applied to 2 x 2 blocks from both sides; sweeps until no rotation is needed
 //   5. eigenvalues ascending, Q = D L^-H V
 // Q overwrites Hs (column-major, eigenvector j in column j), eig ascending; info[p] = 0, or k+1
 // if the equilibrated M is not positive definite at column k.
