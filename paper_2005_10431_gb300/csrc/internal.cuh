@@ -80,7 +80,6 @@ struct MgLevel {
     long long np = 0;
     float* x = nullptr;
     float* b = nullptr;
-    float* t = nullptr;   // work field of a level that coarsens by other than exact halving, else null
 };
 
 struct PendingTiming {

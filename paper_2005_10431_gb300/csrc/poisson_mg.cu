@@ -6,9 +6,8 @@
 //
 // M applies one V-cycle of the second-order (7-point) Laplacian A2 on a hierarchy of grids that
 // halves every dimension while it is even: red-black Gauss-Seidel smoothing, full-weighting
-// restriction of the residual, trilinear prolongation.  Where a dimension is odd and the grid too large for one CTA it
-// coarsens every dimension to a well-divisible number near its half instead (see mg_coarse_dim).  On the coarsest grid (at
-// most 512 points, or up to 16 384 when a dimension turns odd earlier) a fixed number of Chebyshev iterations for the known spectrum of A2 run by one CTA out
+// restriction of the residual, trilinear prolongation, and on the coarsest grid (at most 512
+// points, or up to 16 384 when a dimension turns odd earlier) a fixed number of Chebyshev iterations for the known spectrum of A2 run by one CTA out
 // of shared memory.  A2 and A share their low-frequency spectrum; at the highest grid frequency the
 // order-12 symbol is about 2.5 times the second-order one, so the preconditioned operator M A
 // keeps its eigenvalues in a small interval and AAR reaches a 1e-3 reduction in a few iterations
@@ -150,90 +149,17 @@ __global__ void __launch_bounds__(256) mg_red_kernel(float* __restrict__ x, cons
     x[at(d, p.i, p.j, p.k)] = post_red(x, b, d, p, 1.f / d.diag);
 }
 
-// ---- levels that do not halve exactly ------------------------------------------------------
-// Periodic grids of n and nc points on the same cell: fine point i lies at i nc / n in coarse units, the prolongation is
-// trilinear interpolation there and the restriction its transpose, scaled to keep the mean.  An odd dimension has no red-black
-// colouring, so the smoother is two Jacobi steps with the Chebyshev roots for the upper part [1/3, 2] of the spectrum of
-// D^-1 A2 (damping 0.34, the red-black sweep's is about 0.4).  Bound by launches and L2 like the other levels; six
-// launches a level: 7-point passes of two loads and one store a point, 27 to 125 reads a coarse point in the restriction.
-// The Jacobi scaling that such grids had instead needs 100 to 200 iterations a correction.  Poisson solve, ms: 27^3 4.7 ->
-// 1.4, 45^3 8.7 -> 1.4, 54^3 12.8 -> 1.8, 63^3 16.1 -> 1.7, 82^3 29.6 -> 2.1, 111^3 64.9 -> 3.4.
-constexpr float MG_J0 = 0.5695f, MG_J1 = 1.7319f;   // 1 / (7/6 +- 5/6 cos(pi/4))
-
-// x = J0 b / d, then x + J1 (b - A2 x) / d, which needs b alone
-__global__ void __launch_bounds__(256) mg_any_pre_kernel(float* __restrict__ x, const float* __restrict__ b, MgDims d) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= d.n1 * d.n2 * d.n3) return;
-    const float id = 1.f / d.diag, bt = b[t];
-    const float nb = neighbours(d, point_of(t, d.n1, d.n2), [&](int i, int j, int k) { return b[at(d, i, j, k)]; });
-    x[t] = MG_J0 * id * bt + MG_J1 * id * (bt - MG_J0 * (bt - id * nb));
-}
-// (b - A2 x) at point t
-__device__ __forceinline__ float any_residual(const float* __restrict__ x, const float* __restrict__ b, const MgDims& d, int t) {
-    const float nb = neighbours(d, point_of(t, d.n1, d.n2), [&](int i, int j, int k) { return x[at(d, i, j, k)]; });
-    return b[t] - (d.diag * x[t] - nb);
-}
-// a Jacobi step x + s (b - A2 x), or the residual
-template <bool SWEEP>
-__global__ void __launch_bounds__(256) mg_any_step_kernel(float* __restrict__ out, const float* __restrict__ x,
-                                                          const float* __restrict__ b, MgDims d, float s) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= d.n1 * d.n2 * d.n3) return;
-    const float res = any_residual(x, b, d, t);
-    out[t] = SWEEP ? x[t] + s * res : res;
-}
-// fine points within one coarse spacing of coarse point I along a dimension: [lo, hi], weight 1 - |i nc - I n| / n
-__device__ __forceinline__ int2 any_support(int I, int n, int nc) {
-    const int lo = (I - 1) * n, hi = (I + 1) * n;   // in units of 1 / nc; lo may be negative
-    return make_int2(lo < 0 ? -((-lo) / nc) + ((-lo) % nc == 0 ? 1 : 0) : lo / nc + 1, (hi + nc - 1) / nc - 1);
-}
-__global__ void __launch_bounds__(128) mg_any_restrict_kernel(const float* __restrict__ res, MgDims f,
-                                                              float* __restrict__ bc, MgDims c) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= c.n1 * c.n2 * c.n3) return;
-    const Pt p = point_of(t, c.n1, c.n2);
-    const int2 a = any_support(p.i, f.n1, c.n1), b = any_support(p.j, f.n2, c.n2), g = any_support(p.k, f.n3, c.n3);
-    const float i1 = 1.f / (float)f.n1, i2 = 1.f / (float)f.n2, i3 = 1.f / (float)f.n3;
-    float sum = 0.f;
-    for (int k = g.x; k <= g.y; ++k) {
-        const float wk = 1.f - (float)abs(k * c.n3 - p.k * f.n3) * i3;
-        const int kk = wrapi(k, f.n3);
-        for (int j = b.x; j <= b.y; ++j) {
-            const float wj = wk * (1.f - (float)abs(j * c.n2 - p.j * f.n2) * i2);
-            const float* row = res + (kk * f.n2 + wrapi(j, f.n2)) * f.n1;
-            float s = 0.f;
-            for (int i = a.x; i <= a.y; ++i) s += (1.f - (float)abs(i * c.n1 - p.i * f.n1) * i1) * row[wrapi(i, f.n1)];
-            sum += wj * s;
-        }
-    }
-    bc[t] = sum * ((float)c.n1 * i1) * ((float)c.n2 * i2) * ((float)c.n3 * i3);
-}
-__global__ void __launch_bounds__(256) mg_any_prolong_kernel(float* __restrict__ x, MgDims f, const float* __restrict__ xc,
-                                                             MgDims c) {
-    const int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= f.n1 * f.n2 * f.n3) return;
-    const Pt p = point_of(t, f.n1, f.n2);
-    const int a0 = p.i * c.n1 / f.n1, b0 = p.j * c.n2 / f.n2, c0 = p.k * c.n3 / f.n3;
-    const float u = (float)(p.i * c.n1 - a0 * f.n1) / (float)f.n1, v = (float)(p.j * c.n2 - b0 * f.n2) / (float)f.n2,
-                w = (float)(p.k * c.n3 - c0 * f.n3) / (float)f.n3;
-    const int a1 = wrapi(a0 + 1, c.n1), b1 = wrapi(b0 + 1, c.n2), c1 = wrapi(c0 + 1, c.n3);
-    auto line = [&](int j, int k) { return (1.f - u) * xc[at(c, a0, j, k)] + u * xc[at(c, a1, j, k)]; };
-    x[t] += (1.f - w) * ((1.f - v) * line(b0, c0) + v * line(b1, c0)) + w * ((1.f - v) * line(b0, c1) + v * line(b1, c1));
-}
-
-// The finest level's last half sweep (ANY: last Jacobi step, from w) together with what the AAR iteration does with z = M r: the history push
+// The finest level's last half sweep together with what the AAR iteration does with z = M r: the history push
 // (X = x - x_prev, F = z - z_prev), and either the Richardson step x += omega z or, when an Anderson step follows, z.
-template <bool ANY>
 __global__ void __launch_bounds__(256)
-mg_finish_kernel(float* __restrict__ z, const float* __restrict__ w, const float* __restrict__ b, MgDims d, float* __restrict__ x,
+mg_finish_kernel(float* __restrict__ z, const float* __restrict__ b, MgDims d, float* __restrict__ x,
                  float* __restrict__ xprev, float* __restrict__ zprev, float* __restrict__ Xs, float* __restrict__ Fs,
                  float omega, int have_prev, int richardson) {
     const int t = blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= d.n1 * d.n2 * d.n3) return;
     const Pt p = point_of(t, d.n1, d.n2);
-    const bool red = ANY || ((p.i + p.j + p.k) & 1) == 0;
-    // red points of z are written, black ones read
-    const float zt = ANY ? w[t] + MG_J1 / d.diag * any_residual(w, b, d, t) : red ? post_red(z, b, d, p, 1.f / d.diag) : z[t];
+    const bool red = ((p.i + p.j + p.k) & 1) == 0;
+    const float zt = red ? post_red(z, b, d, p, 1.f / d.diag) : z[t];   // red points of z are written, black ones read
     const float xt = x[t];
     if (have_prev) {
         Xs[t] = xt - xprev[t];
@@ -344,29 +270,15 @@ unsigned mg_blocks(long long work, int bs) { return (unsigned)((work + bs - 1) /
 
 constexpr int MG_COARSE_STOP = 512;    // coarsening stops once a grid has at most this many points
 constexpr int MG_COARSE_MAX = 16384;   // largest coarsest grid (x and d in shared memory)
-// A grid with an odd dimension coarsens to mg_coarse_dim above this size (a coarsest grid of 23^3 or 25^3 points in one CTA
-// made a solve at 46^3 3.7 ms and at 50^3 4.8; 54^3, which coarsens on from 27^3, takes 1.8).  The finest grid does so only above
-// MG_COARSE_MAX: smaller ones keep the Jacobi scaling (25^3 3.5 ms).
-constexpr int MG_ANY_MIN = 4096;
 constexpr size_t MG_TAIL_SMEM = 200 * 1024;   // shared memory of the one-CTA end of the hierarchy
 // its largest swept level: a tail that takes in a 20^3 level costs 34 us; this one 8.6, plus four launches of 2 to 4 us
 constexpr long long MG_TAIL_POINTS = 2048;
 
 }  // namespace
 
-// The coarse size of a dimension of n >= 7 points that is not halved exactly: the number nearest n / 2 that still halves
-// a few times (a multiple of 8 from 48 points on, of 4 from 24, else of 2), between n / 2.4 and n / 1.7
-static int mg_coarse_dim(int n) {
-    const int u = n >= 48 ? 8 : n >= 24 ? 4 : 2;
-    if (n % 2 == 0 && n / 2 % u == 0) return n / 2;
-    const int lo = n / 2 / u * u;
-    return lo >= 2 && n - 2 * lo <= 2 * (lo + u) - n ? lo : lo + u;
-}
-
 // Level hierarchy of the context's grid: level 0 is the fine grid (its x and b are the V-cycle's
 // output and input, supplied per call); each further level halves all three dimensions, until a
-// grid has at most MG_COARSE_STOP points or a dimension is odd; a grid that is then still large
-// (MG_ANY_MIN) coarsens to mg_coarse_dim, and so on.  Returns false (no multigrid)
+// grid has at most MG_COARSE_STOP points or a dimension is odd.  Returns false (no multigrid)
 // unless there is at least one coarse level and the coarsest has at most MG_COARSE_MAX points.
 bool mg_setup(sdft_ctx* c) {
     c->mg.clear();
@@ -377,39 +289,29 @@ bool mg_setup(sdft_ctx* c) {
     }
     L0.np = c->ng;
     std::vector<MgLevel> lv{L0};
-    std::vector<bool> halves;   // level l to l + 1 by exact halving
     while (true) {
         const MgLevel& f = lv.back();
         if (f.np <= MG_COARSE_STOP) break;
         bool even = true;
         for (int d = 0; d < 3; ++d) even = even && f.n[d] % 2 == 0 && f.n[d] >= 4;
-        bool any = f.np > (lv.size() == 1 ? MG_COARSE_MAX : MG_ANY_MIN) && c->ng < (1LL << 30);
-        for (int d = 0; d < 3; ++d) any = any && f.n[d] >= 7;
-        if (!even && !any) break;
+        if (!even) break;
         MgLevel g;
         for (int d = 0; d < 3; ++d) {
-            g.n[d] = even ? f.n[d] / 2 : mg_coarse_dim(f.n[d]);
-            const double q = (double)g.n[d] / f.n[d];
-            g.w[d] = even ? f.w[d] / 4.0 : f.w[d] * q * q;
+            g.n[d] = f.n[d] / 2;
+            g.w[d] = f.w[d] / 4.0;
         }
         g.np = (long long)g.n[0] * g.n[1] * g.n[2];
-        halves.push_back(even);
         lv.push_back(g);
     }
     if (lv.size() < 2 || lv.back().np > MG_COARSE_MAX || c->ng >= (1LL << 30)) return false;
     long long tot = 0;
-    for (size_t l = 0; l < lv.size(); ++l) tot += (l > 0 ? 2 * lv[l].np : 0) + (l + 1 < lv.size() && !halves[l] ? lv[l].np : 0);
+    for (size_t l = 1; l < lv.size(); ++l) tot += 2 * lv[l].np;
     float* buf = (float*)ctx_alloc(c, sizeof(float) * (size_t)tot);
     for (size_t l = 1; l < lv.size(); ++l) {
         lv[l].x = buf;
         lv[l].b = buf + lv[l].np;
         buf += 2 * lv[l].np;
     }
-    for (size_t l = 0; l + 1 < lv.size(); ++l)
-        if (!halves[l]) {
-            lv[l].t = buf;
-            buf += lv[l].np;
-        }
     // coarsest grid: spectrum of the periodic 7-point operator, sum_d 4 w_d sin^2(pi m_d / n_d)
     MgLevel& cl = lv.back();
     double lmax = 0.0, lmin = 1e300;
@@ -429,7 +331,7 @@ bool mg_setup(sdft_ctx* c) {
     // levels from mg_tail on run in one CTA: x and b of each (x, b and the step of the coarsest) in shared memory
     int first = (int)lv.size() - 1;
     size_t smem = sizeof(float) * 3 * (size_t)cl.np;
-    while (first > 1 && (int)lv.size() - first < MG_TAIL && halves[first - 1] && lv[first - 1].np <= MG_TAIL_POINTS &&
+    while (first > 1 && (int)lv.size() - first < MG_TAIL && lv[first - 1].np <= MG_TAIL_POINTS &&
            smem + sizeof(float) * 2 * (size_t)lv[first - 1].np <= MG_TAIL_SMEM) {
         --first;
         smem += sizeof(float) * 2 * (size_t)lv[first].np;
@@ -451,15 +353,6 @@ void mg_enqueue(sdft_ctx* c, const float* r, float* z) {
     auto b = [&](int l) { return l == 0 ? r : (const float*)c->mg[l].b; };
     for (int l = 0; l < tail; ++l) {
         const MgDims d = dims_of(c->mg[l]);
-        if (float* t = c->mg[l].t) {
-            const unsigned nb = mg_blocks(c->mg[l].np, 256);
-            mg_any_pre_kernel<<<nb, 256, 0, c->stream>>>(x(l), b(l), d);
-            mg_any_step_kernel<false><<<nb, 256, 0, c->stream>>>(t, x(l), b(l), d, 0.f);
-            mg_any_restrict_kernel<<<mg_blocks(c->mg[l + 1].np, 128), 128, 0, c->stream>>>(t, d, c->mg[l + 1].b,
-                                                                                          dims_of(c->mg[l + 1]));
-            count_launch(c, 3);
-            continue;
-        }
         mg_pre_kernel<<<mg_blocks(c->mg[l].np, 256), 256, 0, c->stream>>>(x(l), b(l), d);
         mg_restrict_kernel<<<mg_blocks(c->mg[l + 1].np, 128), 128, 0, c->stream>>>(x(l), b(l), d, c->mg[l + 1].b,
                                                                                   dims_of(c->mg[l + 1]));
@@ -486,14 +379,6 @@ void mg_enqueue(sdft_ctx* c, const float* r, float* z) {
     }
     for (int l = tail - 1; l >= 0; --l) {
         const MgDims d = dims_of(c->mg[l]);
-        if (float* t = c->mg[l].t) {
-            const unsigned nb = mg_blocks(c->mg[l].np, 256);
-            mg_any_prolong_kernel<<<nb, 256, 0, c->stream>>>(x(l), d, c->mg[l + 1].x, dims_of(c->mg[l + 1]));
-            mg_any_step_kernel<true><<<nb, 256, 0, c->stream>>>(t, x(l), b(l), d, MG_J0 / d.diag);
-            if (l > 0) mg_any_step_kernel<true><<<nb, 256, 0, c->stream>>>(x(l), t, b(l), d, MG_J1 / d.diag);
-            count_launch(c, l > 0 ? 3 : 2);
-            continue;
-        }
         mg_black_kernel<<<mg_blocks(c->mg[l].np / 2, 128), 128, 0, c->stream>>>(x(l), b(l), d, c->mg[l + 1].x,
                                                                                dims_of(c->mg[l + 1]));
         if (l > 0) mg_red_kernel<<<mg_blocks(c->mg[l].np / 2, 256), 256, 0, c->stream>>>(x(l), b(l), d);
@@ -555,10 +440,8 @@ void mg_residual_vcycle(sdft_ctx* c, const float* x, const float* b, float* r, f
 // the last half sweep of z = M r, the history push and (richardson) the step x += omega z
 void mg_finish(sdft_ctx* c, const float* r, float* z, float* x, float* xprev, float* zprev, float* Xs, float* Fs,
                float omega, bool have_prev, bool richardson) {
-    const float* t = c->mg[0].t;
-    auto kfn = t != nullptr ? mg_finish_kernel<true> : mg_finish_kernel<false>;
-    kfn<<<mg_blocks(c->ng, 256), 256, 0, c->stream>>>(z, t, r, dims_of(c->mg[0]), x, xprev, zprev, Xs, Fs, omega, have_prev,
-                                                      richardson);
+    mg_finish_kernel<<<mg_blocks(c->ng, 256), 256, 0, c->stream>>>(z, r, dims_of(c->mg[0]), x, xprev, zprev, Xs, Fs,
+                                                                  omega, have_prev, richardson);
     SDFT_CUDA(cudaGetLastError());
     count_launch(c);
 }
