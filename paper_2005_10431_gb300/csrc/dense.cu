@@ -214,12 +214,14 @@ gram_reduce_kernel(const double* __restrict__ part, int nsplit, int ncol, double
                     for (int q = 0; q < W; ++q) v[q] += t[1][u][q];
             }
         }
-        if (LANES > 1) {   // an element's lanes are neighbours in one warp and leave the loop together
+        if (LANES > 1) {
+            // exactly the element's lanes: they share o and with it every branch up to here, but not the trip count of the
+            // loop over the terms, so they are named and not taken from whoever is converged
+            const unsigned group = ((1u << (LANES % 32)) - 1u) << ((threadIdx.x & 31) / LANES * LANES);
 #pragma unroll
             for (int off = LANES / 2; off > 0; off >>= 1)
 #pragma unroll
-                for (int q = 0; q < W; ++q)
-                    v[q] += __shfl_down_sync(__activemask(), v[q], off, LANES);
+                for (int q = 0; q < W; ++q) v[q] += __shfl_down_sync(group, v[q], off, LANES);
         }
         if (sub != 0 || j < i) continue;
         const long long ot = (long long)j + (long long)i * ncol;
