@@ -313,10 +313,10 @@ void batched_generalized_eig(sdft_ctx* c, bool cplx, double* const* Ms, double* 
     ScopedTimer timer(c, SDFT_K_EIGEN);
     const size_t sm = geig_smem(n, cplx);
     if (cplx) {
-        SDFT_CUDA(cudaFuncSetAttribute(batched_geig_kernel<Cx>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        allow_dynamic_smem(batched_geig_kernel<Cx>, geig_smem(GEIG_MAX_N, true));
         batched_geig_kernel<Cx><<<count, 256, sm, c->stream>>>(Ms, Hss, eigs, n, info);
     } else {
-        SDFT_CUDA(cudaFuncSetAttribute(batched_geig_kernel<Re>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        allow_dynamic_smem(batched_geig_kernel<Re>, geig_smem(GEIG_MAX_N, false));
         batched_geig_kernel<Re><<<count, 256, sm, c->stream>>>(Ms, Hss, eigs, n, info);
     }
     SDFT_CUDA(cudaGetLastError());

@@ -534,7 +534,7 @@ bool refined_generalized_eig(sdft_ctx* c, const double* M, const double* Hs, dou
     ScopedTimer timer(c, SDFT_K_EIGEN);
     if (n <= RE_MAX_N) {
         const size_t sm = eig32_smem(n);
-        SDFT_CUDA(cudaFuncSetAttribute(eig32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+        allow_dynamic_smem(eig32_kernel, eig32_smem(RE_MAX_N));
         eig32_kernel<<<1, 1024, sm, c->stream>>>(M, Hs, n, X, Lg, status);
     } else {
         // FP32 generalized eigensolve by cuSOLVER on the equilibrated problem (workspace on first use)

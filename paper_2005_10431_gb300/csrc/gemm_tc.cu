@@ -753,8 +753,9 @@ void rotate_tc(sdft_ctx* c, const void* Y, const double* Q, void* X, int ncol) {
         const cuuint32_t box[2] = {64, (cuuint32_t)nj};
         tma_encode_tiled(&mQ, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, Qs, dims, st, box, CU_TENSOR_MAP_SWIZZLE_128B);
     }
-    const size_t dsm = (size_t)NRAW * R_RAW_STAGE + (size_t)NCONV * (R_CONV_A + nj * ROWB) + 1024 + 256;
-    SDFT_CUDA(cudaFuncSetAttribute(rotate_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm));
+    auto smem = [](int cols) { return (size_t)NRAW * R_RAW_STAGE + (size_t)NCONV * (R_CONV_A + cols * ROWB) + 1024 + 256; };
+    const size_t dsm = smem(nj);
+    allow_dynamic_smem(rotate_tc_kernel, smem(R_MAX_NJ));
     const long long ntile = (c->ng + TC_M - 1) / TC_M;
     uint32_t tcols = 32;
     while (tcols < (uint32_t)nj) tcols *= 2;
@@ -793,7 +794,7 @@ void subspace_gram_tc(sdft_ctx* c, const void* Y, const void* HY, double* M, dou
     paired_map(&mY, Y, c->ng, ncol / 2, 16, 64, CU_TENSOR_MAP_SWIZZLE_128B);
     paired_map(&mHY, HY, c->ng, ncol / 2, 16, 64, CU_TENSOR_MAP_SWIZZLE_128B);
     const size_t dsm = (size_t)G_SMEM + 1024 + 256;
-    SDFT_CUDA(cudaFuncSetAttribute(gram_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm));
+    allow_dynamic_smem(gram_tc_kernel, dsm);
     // algorithmic flops: two full ngrid x ncol x ncol products (M and Hs), 2 flops per multiply-add
     ScopedTimer timer(c, SDFT_K_GRAM, 0.0, 4.0 * (double)c->ng * ncol * ncol);
     float* part = reinterpret_cast<float*>(c->part);

@@ -288,6 +288,15 @@ struct sdft_ctx {
 
 namespace sdft {
 
+// Dynamic shared memory of kernel `kfn`: `bound` is what any launch of it may need, on any grid and in any context.  The
+// attribute belongs to the kernel, so a value that followed the launch at hand would be lowered by a context on another
+// host thread between this one's call and its launch, which then fails.
+constexpr int SMEM_OPTIN = 227 * 1024;   // most shared memory of a CTA, static and dynamic
+template <typename K>
+inline void allow_dynamic_smem(K kfn, size_t bound) {
+    SDFT_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bound));
+}
+
 // allocation through the context's callbacks
 void* ctx_alloc(sdft_ctx* c, size_t bytes);
 // release one allocation made by ctx_alloc (stream-ordered through the callbacks, else cudaFree)

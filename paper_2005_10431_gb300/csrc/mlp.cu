@@ -475,7 +475,7 @@ void mlp_loss_grad(const void* feat, const float* target, long long npts, long l
                    const float* params, float* grad, double* loss, cudaStream_t st) {
     SDFT_CUDA(cudaMemsetAsync(grad, 0, sizeof(float) * NP, st));
     const size_t sm = tile_smem(true);
-    SDFT_CUDA(cudaFuncSetAttribute(mlp_tile_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    allow_dynamic_smem(mlp_tile_kernel<true>, sm);
     const long long ntile = (batch + TP - 1) / TP;
     const int grid = (int)std::min<long long>(ntile, tile_grid(st));
     mlp_tile_kernel<true><<<grid, MT, sm, st>>>(reinterpret_cast<const __nv_bfloat16*>(feat), target, npts, batch,
@@ -486,7 +486,7 @@ void mlp_loss_grad(const void* feat, const float* target, long long npts, long l
 
 void mlp_forward(const void* feat, long long npts, const float* params, float* y, cudaStream_t st) {
     const size_t sm = tile_smem(false);
-    SDFT_CUDA(cudaFuncSetAttribute(mlp_tile_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm));
+    allow_dynamic_smem(mlp_tile_kernel<false>, sm);
     const long long ntile = (npts + TP - 1) / TP;
     const int grid = (int)std::min<long long>(ntile, 2LL * tile_grid(st));
     mlp_tile_kernel<false><<<grid, MT, sm, st>>>(reinterpret_cast<const __nv_bfloat16*>(feat), nullptr, npts, npts,

@@ -338,7 +338,7 @@ bool mg_setup(sdft_ctx* c) {
     }
     c->mg_tail = first;
     // the attribute belongs to the kernel, not to this context: allow what any context's tail may need
-    SDFT_CUDA(cudaFuncSetAttribute(mg_tail_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)MG_TAIL_SMEM));
+    allow_dynamic_smem(mg_tail_kernel, MG_TAIL_SMEM);
     c->mg = lv;
     return true;
 }

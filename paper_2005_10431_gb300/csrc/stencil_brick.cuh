@@ -26,6 +26,7 @@ namespace sdft {
 namespace {
 
 constexpr int BRICK_NT = 256;   // at most tw * th threads
+constexpr size_t BRICK_SMEM_MAX = 110 * 1024;   // tile and KB coefficients of a CTA, two CTAs per SM
 
 struct BrickTile {
     int tw, th;          // columns per CTA
@@ -252,7 +253,7 @@ template <typename E, int ZC>
 bool brick_ok(const sdft_ctx* c, int ncolE) {
     return ncolE > 0 && ncolE <= 65535 && (c->n[2] + ZC - 1) / ZC <= 65535 && c->ng < (1LL << 31) &&
            c->opt.boundary == SDFT_BC_PERIODIC &&
-           brick_smem<E>(brick_tile(c->n[0], c->n[1]), ZC, c->natom) <= 110 * 1024;
+           brick_smem<E>(brick_tile(c->n[0], c->n[1]), ZC, c->natom) <= BRICK_SMEM_MAX;
 }
 
 template <typename E, bool CPLX, int ZC, int MINB>
@@ -274,8 +275,7 @@ void launch_brick(sdft_ctx* c, int kpt, const E* Y, const E* Yprev, E* Ynext, in
     ScopedTimer timer(timed ? c : nullptr, sizeof(S) == 8 ? SDFT_K_STENCIL64 : SDFT_K_STENCIL,
                       (double)ncolE * (double)c->ng * sizeof(E) * (prev ? 3.0 : 2.0));
     auto launch = [&](auto kfn) {
-        if (dsm > 48 * 1024)
-            SDFT_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm));
+        if (dsm > 48 * 1024) allow_dynamic_smem(kfn, BRICK_SMEM_MAX);
         kfn<<<grid, nt, dsm, c->stream>>>(Y, Yprev, Ynext, V, kbC, kb.patom, pval, kb.S, t.tw, t.th, t.tiles_x, A);
     };
     if (prev && haskb) launch(brick_kernel<E, CPLX, ZC, MINB, true, true>);

@@ -311,8 +311,7 @@ void chebyshev_filter_multi(const std::vector<sdft_ctx*>& ctxs, const std::vecto
                                       c0->stream));
     auto step = [&](auto kfn, int k) {
         ScopedTimer timer(c0, SDFT_K_STENCIL, elems * sizeof(float2) * (k > 1 ? 3.0 : 2.0));
-        if (dsm > 48 * 1024)
-            SDFT_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm));
+        if (dsm > 48 * 1024) allow_dynamic_smem(kfn, SMEM_OPTIN);
         kfn<<<(unsigned)total, BRICK_NT, dsm, c0->stream>>>(n, k, m, c0->m_steps);
         SDFT_CUDA(cudaGetLastError());
         count_launch(c0);

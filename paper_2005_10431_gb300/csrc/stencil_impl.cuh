@@ -837,8 +837,7 @@ void launch_variant(sdft_ctx* c, int kpt, const E* Y, const E* Yprev, E* Ynext, 
 #define SDFT_STEP(P, K, VV, KN)                                                                      \
     do {                                                                                             \
         auto kfn = cheb_step_kernel<E, CPLX, TX, TY, PF, MINB, D, P, K, VV, KN>;                      \
-        if (dsm > 48 * 1024)                                                                         \
-            SDFT_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm)); \
+        if (dsm > 48 * 1024) allow_dynamic_smem(kfn, SMEM_OPTIN);                                    \
         kfn<<<grid, block, dsm, c->stream>>>(Y, Yprev, Ynext, V, kbC, kb.patom, pval, kb.S, ncolE, A); \
     } while (0)
     SDFT_REQUIRE(kin, SDFT_ERR_INVALID_ARG, "stencil step without kinetic term is not built");
@@ -906,7 +905,7 @@ void launch_row_impl(sdft_ctx* c, int kpt, const float2* Y, const float2* Yprev,
 #define SDFT_ROW(P, KK)                                                                               \
     do {                                                                                              \
         auto kfn = cheb_row_kernel<CPLX, TY, PF, MAXT, MINB, D, P, KK, true>;                          \
-        SDFT_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm));  \
+        allow_dynamic_smem(kfn, SMEM_OPTIN);                                                          \
         kfn<<<grid, block, dsm, c->stream>>>(Y, Yprev, Ynext, V, kbC, kb.patom, kb.pval32, kb.S, A, ncolE, grp); \
     } while (0)
     if (prev && haskb) SDFT_ROW(true, true);

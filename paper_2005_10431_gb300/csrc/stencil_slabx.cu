@@ -35,6 +35,7 @@ constexpr int R = FD_RADIUS;
 constexpr int SX_PFD = 10;              // planes between a stage's copies and the L2 prefetch issued with them
 constexpr int SX_MAXD = 6;              // stages
 constexpr size_t SX_RING = 225 * 1024;
+constexpr size_t SX_TAIL = 16 * SX_MAXD + 128;   // barriers and the ring's alignment
 constexpr int SX_COMP = 320;            // compute threads at most
 constexpr int SX_MAXT = SX_COMP + 32;
 
@@ -377,7 +378,7 @@ SlabxShape slabx_shape(const sdft_ctx* c, int nslot) {
         s.depth = (int)std::min<size_t>(SX_MAXD, SX_RING / s.sstride);
         if (s.depth >= 3 || s.nst <= 1) break;
     }
-    s.smem = (size_t)s.sstride * s.depth + 16 * SX_MAXD + 128;
+    s.smem = (size_t)s.sstride * s.depth + SX_TAIL;
     return s;
 }
 
@@ -447,7 +448,7 @@ void launch_slabx(sdft_ctx* c, int kpt, const float2* Y, const float2* Yprev, fl
     ScopedTimer timer(timed ? c : nullptr, SDFT_K_STENCIL,
                       (double)ncolE * (double)c->ng * sizeof(float2) * (prev ? 3.0 : 2.0));
     auto launch = [&](auto kfn) {
-        SDFT_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)s.smem));
+        allow_dynamic_smem(kfn, SX_RING + SX_TAIL);
         kfn<<<nper * s.nslab, s.nthreads, s.smem, c->stream>>>(Y, Yprev, Ynext, V, kbC, kb.patom, kb.pval32, A,
                                                                stencil_error_flag(c));
     };

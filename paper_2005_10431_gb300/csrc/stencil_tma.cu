@@ -611,7 +611,7 @@ void launch_slab_variant(sdft_ctx* c, int kpt, const float2* Y, const float2* Yp
 #define SDFT_SLAB(P, K, J)                                                                                       \
     do {                                                                                                         \
         auto kfn = cheb_slab_kernel<N1, TY, NP, RY, S, D, MINB, P, K, J>;                                         \
-        SDFT_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm));             \
+        allow_dynamic_smem(kfn, SMEM_OPTIN);                                                                     \
         kfn<<<grid, block, dsm, c->stream>>>(Y, Ynext, kbC, Cn, mfull, m6, mmid, mp, mv, mka, mkv, mq, A, err);    \
     } while (0)
     // fused projection of the output's KB coefficients into the buffer the caller offered
