@@ -24,17 +24,19 @@ struct AtomBox {
 
 // Support points of atom blockIdx.x among chunk blockIdx.y of its box (contiguous in box order): their number into
 // ccnt (FILL false), or, after that, their lists in box order from the sum of the earlier chunks' numbers on.  Bound
-// by the FP64 pipe: the squared displacements of an axis are tabulated once per CTA, so a box point costs three
-// operations, and the normalisation is formed by one thread (a pow() in every thread was half of the time).  One CTA
-// per atom took 146 us for the 64-atom cell, this takes 64 us.
+// by the FP64 pipe: the displacements of an axis are tabulated once per CTA (for boxes whose edges have at most
+// SUP_TABLE points together; longer ones form them at each point), so a box point costs three operations, and the
+// normalisation is formed by one thread (a pow() in every thread was half of the time).  One CTA per atom took 146 us
+// for the 64-atom cell, this takes 64 us.
 constexpr int SUP_CHUNKS = 8;
+constexpr int SUP_TABLE = 6128;   // doubles that fit beside the static arrays in the 48 KB every kernel may have
 template <bool FILL>
 __global__ void __launch_bounds__(256)
 atom_support_kernel(const AtomBox* __restrict__ boxes, int cap, int n1, int n2, int n3, double h1, double h2, double h3,
                     double k1, double k2, double k3, int cplx, int* __restrict__ ccnt, int* __restrict__ cnt,
                     int* __restrict__ idx, int* __restrict__ img, double* __restrict__ val64,
-                    float* __restrict__ val32, int isolated) {
-    extern __shared__ double disp[];   // displacements of the box's columns, rows and planes
+                    float* __restrict__ val32, int isolated, int tabulated) {
+    extern __shared__ double disp[];   // displacements of the box's columns, rows and planes (tabulated)
     const int a = blockIdx.x;
     const AtomBox B = boxes[a];
     const int total = B.dim[0] * B.dim[1] * B.dim[2];
@@ -45,9 +47,15 @@ atom_support_kernel(const AtomBox* __restrict__ boxes, int cap, int n1, int n2, 
     double* const dx = disp;
     double* const dy = dx + B.dim[0];
     double* const dz = dy + B.dim[1];
-    for (int i = threadIdx.x; i < B.dim[0]; i += blockDim.x) dx[i] = (B.lo[0] + i) * h1 - B.pos[0];
-    for (int i = threadIdx.x; i < B.dim[1]; i += blockDim.x) dy[i] = (B.lo[1] + i) * h2 - B.pos[1];
-    for (int i = threadIdx.x; i < B.dim[2]; i += blockDim.x) dz[i] = (B.lo[2] + i) * h3 - B.pos[2];
+    auto displacement = [&](int d, int i) {
+        const double h = d == 0 ? h1 : d == 1 ? h2 : h3;
+        return fma((double)(B.lo[d] + i), h, -B.pos[d]);
+    };
+    if (tabulated) {
+        for (int i = threadIdx.x; i < B.dim[0]; i += blockDim.x) dx[i] = displacement(0, i);
+        for (int i = threadIdx.x; i < B.dim[1]; i += blockDim.x) dy[i] = displacement(1, i);
+        for (int i = threadIdx.x; i < B.dim[2]; i += blockDim.x) dz[i] = displacement(2, i);
+    }
     if (threadIdx.x == 0) {
         base = 0;
         if (FILL) {
@@ -75,7 +83,9 @@ atom_support_kernel(const AtomBox* __restrict__ boxes, int cap, int n1, int n2, 
             I[0] = B.lo[0] + ix;
             I[1] = B.lo[1] + iy;
             I[2] = B.lo[2] + iz;
-            r2 = fma(dz[iz], dz[iz], fma(dx[ix], dx[ix], __dmul_rn(dy[iy], dy[iy])));
+            const double x = tabulated ? dx[ix] : displacement(0, ix), y = tabulated ? dy[iy] : displacement(1, iy),
+                         z = tabulated ? dz[iz] : displacement(2, iz);
+            r2 = fma(z, z, fma(x, x, __dmul_rn(y, y)));
             keep = r2 < B.rc * B.rc;
             // an isolated cell has no periodic images: points beyond the grid are not wrapped back in
             if (isolated && (I[0] < 0 || I[0] >= n1 || I[1] < 0 || I[1] >= n2 || I[2] < 0 || I[2] >= n3)) keep = false;
@@ -246,14 +256,13 @@ void build_kb_tables(sdft_ctx* c, int kpt) {
         SDFT_CUDA(cudaMemcpyAsync(dboxes, boxes.data(), sizeof(AtomBox) * c->natom, cudaMemcpyHostToDevice, c->stream));
         int side = 0;
         for (const AtomBox& B : boxes) side = std::max(side, B.dim[0] + B.dim[1] + B.dim[2]);
-        const size_t dsm = sizeof(double) * (size_t)side;
+        const bool tabulated = side <= SUP_TABLE;
+        const size_t dsm = tabulated ? sizeof(double) * (size_t)side : 0;
         auto launch = [&](auto kfn) {
-            if (dsm > 48 * 1024)
-                SDFT_CUDA(cudaFuncSetAttribute(kfn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)dsm));
             kfn<<<dim3(c->natom, SUP_CHUNKS), 256, dsm, c->stream>>>(dboxes, T.cap, c->n[0], c->n[1], c->n[2], c->h[0],
                                                                      c->h[1], c->h[2], kred[0], kred[1], kred[2],
                                                                      T.cplx, ccnt, T.cnt, T.idx, T.img, T.val64,
-                                                                     T.val32, c->opt.boundary == SDFT_BC_DIRICHLET);
+                                                                     T.val32, c->opt.boundary == SDFT_BC_DIRICHLET, tabulated);
         };
         launch(atom_support_kernel<false>);
         launch(atom_support_kernel<true>);
