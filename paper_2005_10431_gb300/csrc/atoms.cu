@@ -160,6 +160,7 @@ atom_field_kernel(const AtomA* __restrict__ at, int natom, const __grid_constant
 // f_c = sin^2(pi (rc - r) / (2 rc)) carry FP32 rounding only, as the sums do.  Bound by the 32 exponentials
 // per point and atom within 6.5 bohr (special function unit).  64-atom cell, 80^3: 4465 -> 100 us.
 constexpr int NDESC = 32;
+constexpr double DESC_RC = 6.5;
 // 2^x by the special function unit (2 ulp, as exp2f), results below 2^-126 flushed to 0
 __device__ __forceinline__ float exp2_approx(float x) {
     float y;
@@ -278,29 +279,59 @@ overlap_energy_kernel(const PairAtom* __restrict__ at, int natom, int m1, int m2
     }
 }
 
+// Bytes of the axis tables of natom atoms cut off at `cut`, after their AtomA; M: image slots per atom and axis
+size_t axis_bytes(const sdft_ctx* c, double cut, bool iso, int (&M)[3], long long (&size)[3]) {
+    long long total = 0;
+    for (int d = 0; d < 3; ++d) {
+        // at most floor(2 cut / L) + 1 integers lie in an interval of length 2 cut / L
+        M[d] = iso ? 1 : (int)std::floor(2.0 * cut / c->L[d]) + 1;
+        size[d] = (long long)c->natom * M[d] * c->n[d];
+        total += size[d];
+    }
+    return sizeof(AtomA) * (size_t)c->natom + 256 + sizeof(double2) * (size_t)total;
+}
+
+int overlap_chunks(int natom) { return std::max(1, std::min(16, (8 * 152 + natom - 1) / natom)); }
+size_t overlap_bytes(int natom) {
+    return sizeof(PairAtom) * (size_t)natom + 256 + sizeof(double) * 4 * (size_t)natom * overlap_chunks(natom);
+}
+
+// The context's buffer for the tables below: its size follows from the cell, the grid and the species, not from the
+// positions, so it is allocated once, at creation, and no later call allocates or releases memory for them.
+void reserve_atom_tables(sdft_ctx* c) {
+    if (c->atom_tab) return;
+    int M[3];
+    long long size[3];
+    double cut = 0.0;
+    for (const sdft_pseudo& s : c->species) cut = std::max(cut, 10.0 * std::max(s.r_loc, s.sad_width));
+    size_t bytes = overlap_bytes(c->natom);
+    bytes = std::max(bytes, axis_bytes(c, cut, c->opt.boundary == SDFT_BC_DIRICHLET, M, size));
+    bytes = std::max(bytes, axis_bytes(c, DESC_RC, false, M, size));
+    c->atom_tab = ctx_alloc(c, bytes);
+    c->atom_tab_bytes = bytes;
+}
+// `first` elements of A, then an array of B, in that buffer
+template <typename A, typename B>
+void atom_tables(sdft_ctx* c, size_t first, A*& a, B*& b) {
+    a = reinterpret_cast<A*>(c->atom_tab);
+    b = reinterpret_cast<B*>(static_cast<char*>(c->atom_tab) + (sizeof(A) * first + 255) / 256 * 256);
+}
+
 inline unsigned nb(long long n) { return (unsigned)std::min<long long>((n + 255) / 256, 152LL * 16); }
 
-// the three axis tables for atoms with positions, widths and cut-offs `at` (device copy in *dat); both stay
-// allocated until drop()
+// the three axis tables for atoms with positions, widths and cut-offs `at` (device copy in *dat), in the context's buffer
+// until the next use of it
 struct AxisWork {
-    sdft_ctx* c;
     AtomA* dat = nullptr;
-    double2* tab = nullptr;
     AxisTables T;
-    AxisWork(sdft_ctx* c_, const std::vector<AtomA>& at, bool iso, bool separable) : c(c_) {
+    AxisWork(sdft_ctx* c, const std::vector<AtomA>& at, bool iso, bool separable) {
         double cut = 0.0;
         for (const AtomA& a : at) cut = std::max(cut, a.cut);
-        long long size[3], total = 0;
-        for (int d = 0; d < 3; ++d) {
-            // at most floor(2 cut / L) + 1 integers lie in an interval of length 2 cut / L
-            T.M[d] = iso ? 1 : (int)std::floor(2.0 * cut / c->L[d]) + 1;
-            size[d] = (long long)at.size() * T.M[d] * c->n[d];
-            total += size[d];
-        }
-        dat = (AtomA*)ctx_alloc(c, sizeof(AtomA) * at.size());
-        tab = (double2*)ctx_alloc(c, sizeof(double2) * total);
+        long long size[3];
+        SDFT_REQUIRE(axis_bytes(c, cut, iso, T.M, size) <= c->atom_tab_bytes, SDFT_ERR_INVALID_ARG, "atom tables too large");
+        double2* p = nullptr;
+        atom_tables(c, at.size(), dat, p);
         SDFT_CUDA(cudaMemcpyAsync(dat, at.data(), sizeof(AtomA) * at.size(), cudaMemcpyHostToDevice, c->stream));
-        double2* p = tab;
         for (int d = 0; d < 3; ++d) {
             T.t[d] = p;
             axis_table_kernel<<<nb(size[d]), 256, 0, c->stream>>>(dat, (int)at.size(), d, T.M[d], c->n[d], c->h[d],
@@ -309,10 +340,6 @@ struct AxisWork {
         }
         SDFT_CUDA(cudaGetLastError());
         count_launch(c, 3);
-    }
-    void drop() {
-        ctx_release(c, tab);
-        ctx_release(c, dat);
     }
 };
 
@@ -331,6 +358,7 @@ inline int row_threads(int n1) { return std::min(ROW_MAXT, (n1 + 31) / 32 * 32);
 void build_pseudocharge_and_sad(sdft_ctx* c) {
     const int nt = row_threads(c->n[0]);
     const unsigned grid = (unsigned)(c->n[1] * c->n[2]);
+    reserve_atom_tables(c);
     // Below 2^15 points the direct sums stay (24^3 points, 2 atoms: 110 us direct, 36 us separable; 40^3 points, 8 atoms:
     // 343 and 49; 48^3 points, 8 atoms: 310 and 50), although they cost more, so that a small cell's fields stay the same
     // bit for bit: an unconverged FP64 SCF started from random orbitals turns a last-bit change of its density into
@@ -351,7 +379,6 @@ void build_pseudocharge_and_sad(sdft_ctx* c) {
         else atom_field_kernel<false><<<grid, nt, 0, c->stream>>>(W.dat, c->natom, W.T, c->n[0], c->n[1], c->n[2], out);
         SDFT_CUDA(cudaGetLastError());
         count_launch(c);
-        W.drop();
     }
     // normalise the SAD density to N_e: sum rho = rho . 1
     double* ones = c->work64;
@@ -367,7 +394,7 @@ void build_pseudocharge_and_sad(sdft_ctx* c) {
 
 // descriptors of every grid point, BF16 [ng][32] (the network's cut-off radius is 6.5 bohr)
 void descriptor_field(sdft_ctx* c, void* feat) {
-    const double rc = 6.5;
+    const double rc = DESC_RC;
     std::vector<AtomA> at = atom_table(c);
     for (AtomA& a : at) {
         a.amp = 1.0;
@@ -380,7 +407,6 @@ void descriptor_field(sdft_ctx* c, void* feat) {
         W.dat, c->natom, W.T, c->n[0], c->n[1], c->n[2], (float)rc, reinterpret_cast<__nv_bfloat16*>(feat));
     SDFT_CUDA(cudaGetLastError());
     count_launch(c);
-    W.drop();
 }
 
 // E_self = sum Z^2 / (2 sqrt(pi) r_loc) and the overlap correction with its gradient (host results)
@@ -396,9 +422,11 @@ void energy_constants(sdft_ctx* c) {
     const double rmax = 30.0;
     int m[3];
     for (int d = 0; d < 3; ++d) m[d] = c->opt.boundary == SDFT_BC_DIRICHLET ? 0 : (int)std::ceil(rmax / c->L[d]) + 1;
-    const int nchunk = std::max(1, std::min(16, (8 * 152 + na - 1) / na));
-    PairAtom* dat = (PairAtom*)ctx_alloc(c, sizeof(PairAtom) * na);
-    double* dout = (double*)ctx_alloc(c, sizeof(double) * 4 * na * nchunk);
+    const int nchunk = overlap_chunks(na);
+    reserve_atom_tables(c);
+    PairAtom* dat;
+    double* dout;
+    atom_tables(c, na, dat, dout);
     SDFT_CUDA(cudaMemcpyAsync(dat, at.data(), sizeof(PairAtom) * na, cudaMemcpyHostToDevice, c->stream));
     overlap_energy_kernel<<<dim3(na, nchunk), 256, 0, c->stream>>>(dat, na, m[0], m[1], m[2], c->L[0], c->L[1], c->L[2],
                                                                    rmax, dout);
@@ -407,8 +435,6 @@ void energy_constants(sdft_ctx* c) {
     std::vector<double> out((size_t)4 * na * nchunk);
     SDFT_CUDA(cudaMemcpyAsync(out.data(), dout, sizeof(double) * out.size(), cudaMemcpyDeviceToHost, c->stream));
     SDFT_CUDA(cudaStreamSynchronize(c->stream));
-    ctx_release(c, dout);
-    ctx_release(c, dat);
     c->E_sc = 0.0;
     c->dEsc.assign(3 * (size_t)na, 0.0);
     for (int a = 0; a < na; ++a)

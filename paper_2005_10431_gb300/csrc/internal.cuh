@@ -199,6 +199,8 @@ struct sdft_ctx {
     double* veff = nullptr;       // [nspin][ng]
     float* veff32 = nullptr;      // [nspin][ng]
     double* exc = nullptr;        // eps_xc
+    void* atom_tab = nullptr;     // per-atom and per-axis tables of atoms.cu (allocated at creation, large enough for all)
+    size_t atom_tab_bytes = 0;
     double* work64 = nullptr;     // [28*ng] grid scratch (Poisson, mixing, energies, Lanczos)
     float* work32 = nullptr;      // [20*ng] FP32 scratch of the mixed-precision Poisson solver
     // small device scalars / reductions [SCAL_DOUBLES], regions:
