@@ -78,11 +78,14 @@ def sdft_default_options(**overrides) -> sdft_options:
 
 
 def _torch_allocator(device):
+    """Allocation callbacks over torch's caching allocator.  `user` is the context's stream: a block that the context
+    gives back while its kernels still run may be handed out again only to work behind them, so it has to come from
+    that stream's pool, whichever stream is current at the call."""
     import torch
 
     def alloc(nbytes, user):
         try:
-            return torch.cuda.caching_allocator_alloc(int(nbytes), device=device)
+            return torch.cuda.caching_allocator_alloc(int(nbytes), device=device, stream=int(user or 0))
         except Exception:
             return None
 
@@ -132,8 +135,8 @@ def sdft_create(L, n, pos, types, species, options: dict | None = None, kpts=Non
         af, ff = _lib.ALLOC_FN(), _lib.FREE_FN()
     keep += [af, ff]
     h = C.c_void_p()
-    code = L_.sdft_create(C.byref(cell), C.byref(grid), C.byref(atoms), len(species), sp, C.byref(o), af, ff, None,
-                          C.c_void_p(stream_handle), C.byref(h))
+    code = L_.sdft_create(C.byref(cell), C.byref(grid), C.byref(atoms), len(species), sp, C.byref(o), af, ff,
+                          C.c_void_p(stream_handle), C.c_void_p(stream_handle), C.byref(h))
     _check(code, None)
     cplx = [bool(np.any(k[i] != 0)) for i in range(o.nkpt)]
     return Context(h, keep, o.nspin, o.nkpt, o.nstates, int(np.prod(n)), pos.shape[0], o.precision, cplx)

@@ -80,3 +80,25 @@ def test_moves_keep_the_number_of_blocks(sd, monkeypatch):
     # the projector tables (six by atom, four by point) and their three scratch blocks
     assert asked == [13, 13, 13]
     sd.sdft_destroy(ctx)
+
+
+@pytest.mark.parametrize("current", [False, True])
+def test_blocks_belong_to_the_contexts_stream(sd, monkeypatch, current):
+    # a block released while the context's kernels run must not reach another stream's work
+    make, streams = torch.cuda.caching_allocator_alloc, []
+
+    def seen(size, device=None, stream=None):
+        streams.append(torch.cuda.current_stream().cuda_stream if stream is None else getattr(stream, "cuda_stream", stream))
+        return make(size, device, stream)
+
+    monkeypatch.setattr(torch.cuda, "caching_allocator_alloc", seen)
+    own = torch.cuda.Stream()
+    cell = workloads.small_cell(npts=12, L=4.0, natom=2, seed=3, nstates=8)
+    with torch.cuda.stream(own if current else torch.cuda.default_stream()):
+        ctx = sd.sdft_create(cell.L, cell.n, cell.pos, cell.types, cell.species, dict(nstates=8, precision=sd.SDFT_FP64),
+                             stream=None if current else own)
+    created = len(streams)
+    sd.sdft_move_atoms(ctx, cell.pos, 0)   # under the default stream in either case
+    assert len(streams) > created > 0
+    assert set(streams) == {own.cuda_stream}
+    sd.sdft_destroy(ctx)
