@@ -224,6 +224,34 @@ void chebyshev_filter_multi(const std::vector<sdft_ctx*>& ctxs, const std::vecto
     const int n = (int)ctxs.size();
     SDFT_REQUIRE(m >= 1, SDFT_ERR_INVALID_ARG, "degree must be >= 1");
     SDFT_REQUIRE(n >= 1 && n <= MULTI_MAX, SDFT_ERR_INVALID_ARG, "multi-cell launch takes 1..64 cells");
+    for (int i = 0; i < n; ++i)
+        SDFT_REQUIRE(b[i] > a[i] && a[i] > a0[i], SDFT_ERR_INVALID_ARG, "filter bounds must satisfy a0 < a < b");
+    // cells whose KB coefficients do not fit beside a brick (some 5000 atoms and more) are filtered on their own
+    std::vector<int> fit;
+    for (int i = 0; i < n; ++i)
+        if (brick_ok<float2, MULTI_ZC>(ctxs[i], ctxs[i]->nfilt / 2)) fit.push_back(i);
+    if ((int)fit.size() < n) {
+        std::vector<sdft_ctx*> cs;
+        std::vector<const void*> xs;
+        std::vector<void*> ys;
+        std::vector<double> as, bs, a0s;
+        for (int i = 0, q = 0; i < n; ++i) {
+            if (q < (int)fit.size() && fit[q] == i) {
+                ++q;
+                cs.push_back(ctxs[i]);
+                xs.push_back(X[i]);
+                ys.push_back(Y[i]);
+                as.push_back(a[i]);
+                bs.push_back(b[i]);
+                a0s.push_back(a0[i]);
+            } else {
+                sdft_ctx* c = ctxs[i];
+                chebyshev_filter(c, 0, SDFT_MIXED, X[i], Y[i], c->nfilt, m, a[i], b[i], a0[i], c->veff, c->veff32);
+            }
+        }
+        if (!cs.empty()) chebyshev_filter_multi(cs, xs, ys, m, as.data(), bs.data(), a0s.data());
+        return;
+    }
     sdft_ctx* c0 = ctxs[0];
     // per cell: grid, tile, ring of its own block buffers (T1, T2, Y), recurrence scalars of every step
     std::vector<MultiProblem> probs(n);
@@ -233,7 +261,6 @@ void chebyshev_filter_multi(const std::vector<sdft_ctx*>& ctxs, const std::vecto
     double elems = 0;
     for (int i = 0; i < n; ++i) {
         sdft_ctx* c = ctxs[i];
-        SDFT_REQUIRE(b[i] > a[i] && a[i] > a0[i], SDFT_ERR_INVALID_ARG, "filter bounds must satisfy a0 < a < b");
         const double e = 0.5 * (b[i] - a[i]), cc = 0.5 * (b[i] + a[i]);
         const double sigma1 = e / (a0[i] - cc);
         double sigma = sigma1;
@@ -311,7 +338,7 @@ void chebyshev_filter_multi(const std::vector<sdft_ctx*>& ctxs, const std::vecto
                                       c0->stream));
     auto step = [&](auto kfn, int k) {
         ScopedTimer timer(c0, SDFT_K_STENCIL, elems * sizeof(float2) * (k > 1 ? 3.0 : 2.0));
-        if (dsm > 48 * 1024) allow_dynamic_smem(kfn, SMEM_OPTIN);
+        if (dsm > 48 * 1024) allow_dynamic_smem(kfn, BRICK_SMEM_MAX);
         kfn<<<(unsigned)total, BRICK_NT, dsm, c0->stream>>>(n, k, m, c0->m_steps);
         SDFT_CUDA(cudaGetLastError());
         count_launch(c0);
