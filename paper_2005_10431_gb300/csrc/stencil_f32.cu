@@ -320,14 +320,20 @@ void chebyshev_filter_multi(const std::vector<sdft_ctx*>& ctxs, const std::vecto
             ktab.push_back(KBProblem{cur, c->C32, kb.cnt, kb.idx, kb.val32, kb.gamma, kb.cap, kb.natom, c->nfilt / 2,
                                      c->ng});
         }
-    if (c0->m_ktab_cap < (int)ktab.size()) {
-        c0->m_ktab = (KBProblem*)ctx_alloc(c0, sizeof(KBProblem) * ktab.size());
-        c0->m_ktab_cap = (int)ktab.size();
-    }
-    if (c0->m_steps_cap < m * n) {
-        c0->m_steps = (float2*)ctx_alloc(c0, sizeof(float2) * m * n);
-        c0->m_steps_cap = m * n;
-    }
+    // the tables grow with degree and cells; an outgrown one is given back once nothing reads it any more
+    auto grow = [&](auto*& table, int& cap, int need) {
+        if (cap >= need) return;
+        if (table) {
+            SDFT_CUDA(cudaStreamSynchronize(c0->stream));
+            ctx_release(c0, table);
+            table = nullptr;
+            cap = 0;
+        }
+        table = reinterpret_cast<std::remove_reference_t<decltype(table)>>(ctx_alloc(c0, sizeof(*table) * (size_t)need));
+        cap = need;
+    };
+    grow(c0->m_ktab, c0->m_ktab_cap, (int)ktab.size());
+    grow(c0->m_steps, c0->m_steps_cap, m * n);
     // pageable sources: the copies are staged before the calls return, so the vectors may go out of scope
     if (nk > 0)
         SDFT_CUDA(cudaMemcpyAsync(c0->m_ktab, ktab.data(), sizeof(KBProblem) * ktab.size(), cudaMemcpyHostToDevice,

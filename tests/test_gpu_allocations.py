@@ -1,5 +1,6 @@
 """What a context asks of its allocator: nothing for the descriptors of a learned start beyond the scratch that
-sdft_mlp_predict documents, and nothing more for moved atoms than the projector tables take."""
+sdft_mlp_predict documents; nothing more for moved atoms than the projector tables take; and
+tables of a multi-cell filter that do not pile up as cells and degrees grow."""
 import pytest
 
 pytestmark = pytest.mark.gpu
@@ -80,6 +81,25 @@ def test_moves_keep_the_number_of_blocks(sd, monkeypatch):
     # the projector tables (six by atom, four by point) and their three scratch blocks
     assert asked == [13, 13, 13]
     sd.sdft_destroy(ctx)
+
+
+def test_tables_of_growing_filters_are_replaced(sd, monkeypatch):
+    count = Counter(sd, monkeypatch)
+    cells, ctxs, xs = [], [], []
+    for i in range(4):
+        cell, ctx = _ctx(sd, 12, 2, sd.SDFT_MIXED)
+        sd.sdft_set_veff(ctx, 0, torch.zeros(cell.ngrid, dtype=torch.float64, device="cuda"))
+        cells.append(cell)
+        ctxs.append(ctx)
+        xs.append(sd.pack_block(workloads.initial_orbitals(i, cell.ngrid, cell.nstates), sd.SDFT_MIXED))
+    ys = [torch.empty_like(x) for x in xs]
+    before = len(count.live)
+    for n, degree in ((1, 2), (2, 3), (4, 5), (4, 9), (2, 30), (3, 4)):
+        sd.sdft_chebyshev_filter_multi(ctxs[:n], xs[:n], ys[:n], degree, [3.0] * n, [90.0] * n, [-1.0] * n)
+        assert len(count.live) == before + 2   # the projections' problems and the steps' scalars
+    for ctx in ctxs:
+        sd.sdft_destroy(ctx)
+    assert not count.live
 
 
 @pytest.mark.parametrize("current", [False, True])
