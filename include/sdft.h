@@ -422,7 +422,8 @@ sdft_status sdft_reset_kernel_stats(sdft_ctx* ctx);
  *   Parameters: one FP32 vector of SDFT_MLP_NPARAM: W1 [64 x 32] row-major, b1 [64],
  *     W2 [64 x 64] row-major, b2 [64], w3 [64], b3.  Kernels round the parameters to BF16 and
  *     compute in FP32 (training keeps the FP32 vector as the master copy).
- *   Features: device BF16 (uint16 bit patterns) [npts][32], point-major.
+ *   Features: device BF16 (uint16 bit patterns) [npts][32], point-major; a value that the library
+ *     computes is within 0.51 units of its last BF16 place of the exact sum (subnormal ones too).
  *   Loss: mean over the batch of (y - t)^2.
  *   Mini-batches: the batch of size B starting at s visits points perm((s + i) mod npts), i < B,
  *     with perm(j) = j * P mod npts, P = 1000003 (999983 when 1000003 divides npts).

@@ -155,21 +155,34 @@ atom_field_kernel(const AtomA* __restrict__ at, int natom, const __grid_constant
 }
 
 // Radial descriptors G_q = sum exp(-(r - mu_q)^2 / (2 eta^2)) f_c(r), mu_q = q eta, eta = 6/31, of every
-// grid point, in BF16 [ng][32].  The squared distance is FP64; r = hi + lo in two FP32 words (FP32 square
-// root, corrected by the FP64 remainder), so the Gaussians' arguments and the cut-off function
-// f_c = sin^2(pi (rc - r) / (2 rc)) carry FP32 rounding only, as the sums do.  Bound by the 32 exponentials
-// per point and atom within 6.5 bohr (special function unit).  64-atom cell, 80^3: 4465 -> 100 us.
+// grid point, in BF16 [ng][32].  The squared distance is FP64; r = hi + lo in two FP32 words (FP32 square root, corrected
+// by the FP64 remainder), and the Gaussians' arguments and that of the cut-off function f_c = sin^2(pi (rc - r) / (2 rc))
+// keep both words until their last operation.  Against 64-bit sums (cells of 24^3 to 40^3 points) 1.0e-4 to 2.5e-4 of the
+// values are rounded to the wrong BF16 neighbour; an FP64 square root and cosine with FP32 distances and exponentials,
+// which this replaced, gave 2.5e-4 to 5.9e-4.  Bound by the 32 exponentials per point and atom within 6.5 bohr (issue
+// and special function unit).  64-atom cell, 80^3: 4480 -> 152 us; with arguments of one FP32 word and results below
+// 2^-126 flushed it took 131 us, misrounded 3.5e-4 to 9.3e-4 and lost half of BF16's subnormal values.
 constexpr int NDESC = 32;
 constexpr double DESC_RC = 6.5;
-// 2^x by the special function unit (2 ulp, as exp2f), results below 2^-126 flushed to 0
+// 2^x by the special function unit (2 ulp, as exp2f; results below 2^-126 are kept: BF16 holds values down to 2^-133)
 __device__ __forceinline__ float exp2_approx(float x) {
     float y;
-    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    asm("ex2.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
     return y;
+}
+// sin^2(pi x), x = (rc - r) / (2 rc) in [0, 1/2], for r = hi + lo: x = xh + xl, sin(pi x) = sin(pi xh) + pi xl cos(pi xh)
+// (the cosine, to a few digits, from its Taylor series)
+__device__ __forceinline__ float cutoff(float hi, float lo) {
+    constexpr float RC = (float)DESC_RC, K = 0.5f / RC, K_LO = (float)(0.5 / DESC_RC - (double)K);
+    const float y = RC - hi, yl = ((RC - y) - hi) - lo;
+    const float xh = y * K, xl = fmaf(yl, K, fmaf(y, K_LO, fmaf(y, K, -xh)));
+    const float x2 = xh * xh, c = fmaf(x2, fmaf(x2, fmaf(x2, -1.33526f, 4.05871f), -4.93480f), 1.f);
+    const float s = fmaf(3.14159265f * xl, c, sinpif(xh));
+    return s * s;
 }
 __global__ void __launch_bounds__(ROW_MAXT)
 descriptor_row_kernel(const AtomA* __restrict__ at, int natom, const __grid_constant__ AxisTables T, int n1, int n2,
-                      int n3, float rc, __nv_bfloat16* __restrict__ feat) {
+                      int n3, __nv_bfloat16* __restrict__ feat) {
     __shared__ RowList S;
     const int k = blockIdx.x / n2, j = blockIdx.x - k * n2;   // the CTA's row
     const int ncand = natom * T.M[2] * T.M[1];
@@ -190,14 +203,17 @@ descriptor_row_kernel(const AtomA* __restrict__ at, int natom, const __grid_cons
                         const double r2 = d2 + s;
                         const float hi = sqrtf((float)r2);
                         const float lo = hi > 0.f ? (float)fma(-(double)hi, (double)hi, r2) * (0.5f / hi) : 0.f;
-                        const float sc = sinpif(((rc - hi) - lo) * (0.5f / rc));
-                        const float fc = sc * sc;
-                        // u_q = (r - mu_q) / eta = r 31/6 - q; exp(-u^2 / 2) = 2^(-u^2 log2(e) / 2)
-                        const float t = fmaf(lo, 31.f / 6.f, hi * (31.f / 6.f));
+                        const float fc = cutoff(hi, lo);
+                        // u_q = (r - mu_q) / eta = r 31/6 - q; exp(-u^2 / 2) = 2^(-w^2), w = u sqrt(log2(e) / 2).  r 31/6
+                        // as its nearest integer and the rest, so that w is rounded once, relative to itself
+                        constexpr float C = 31.f / 6.f, C_LO = (float)(31.0 / 6.0 - (double)C);
+                        const float t = hi * C, tl = fmaf(lo, C, fmaf(hi, C_LO, fmaf(hi, C, -t)));
+                        constexpr float SK = 0.84932180028801904f;
+                        const float ti = rintf(t), wf = ((t - ti) + tl) * SK;
 #pragma unroll
                         for (int q = 0; q < NDESC; ++q) {
-                            const float u = t - (float)q;
-                            G[q] = fmaf(exp2_approx(u * u * -0.72134752044448170f), fc, G[q]);
+                            const float w = fmaf(ti - (float)q, SK, wf);
+                            G[q] = fmaf(exp2_approx(-w * w), fc, G[q]);
                         }
                     }
                 }
@@ -394,17 +410,16 @@ void build_pseudocharge_and_sad(sdft_ctx* c) {
 
 // descriptors of every grid point, BF16 [ng][32] (the network's cut-off radius is 6.5 bohr)
 void descriptor_field(sdft_ctx* c, void* feat) {
-    const double rc = DESC_RC;
     std::vector<AtomA> at = atom_table(c);
     for (AtomA& a : at) {
         a.amp = 1.0;
         a.w = 1.0;
-        a.cut = rc;
+        a.cut = DESC_RC;
     }
     // images on the periodic lattice whatever the boundary condition, as the network was trained
     AxisWork W(c, at, false, true);
     descriptor_row_kernel<<<(unsigned)(c->n[1] * c->n[2]), row_threads(c->n[0]), 0, c->stream>>>(
-        W.dat, c->natom, W.T, c->n[0], c->n[1], c->n[2], (float)rc, reinterpret_cast<__nv_bfloat16*>(feat));
+        W.dat, c->natom, W.T, c->n[0], c->n[1], c->n[2], reinterpret_cast<__nv_bfloat16*>(feat));
     SDFT_CUDA(cudaGetLastError());
     count_launch(c);
 }
