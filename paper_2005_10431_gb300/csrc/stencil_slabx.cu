@@ -15,6 +15,8 @@
 //   * V_eff and KB rows (4-byte values, n1 even) start on an 8-byte boundary: their copies start up to two values early,
 //     and the reader skips them;
 //   * KB slots past the staged ones are read from L2 by the few points that have them.
+//   * the diagonal of the kinetic term and V_eff are added last.  Added first, as the largest term, they set the rounding
+//     of the 24 sums that follow: H X was off by 1.27e-7 (root mean square, relative), 0.59e-7 now, column tile 0.80e-7.
 // TY is what 320 compute threads hold (11 warps of 168 registers): 2 floor(640 / n1) rows, evened out over the slabs.
 // Measured, us per step (best of the other tiles -> this one): 82 x 82 x 76, 176 columns 706 -> 358 (at 100 % of the
 // copy bandwidth 160); 96^3, 300 columns 1600 -> 915 (471); 64 x 60 x 60, 66 columns 115 -> 63 (27).  Latency of the few
@@ -270,14 +272,6 @@ cheb_slabx_kernel(const float2* __restrict__ Y, const float2* __restrict__ Yprev
                                 if (st1) slabx_kb_far(st + cofs, g + (unsigned)n1, patom, pval, A, s10, s11);
                             }
                         }
-                        {
-                            const uint32_t va = st + A.off_v + ((g0 + A.vmis) & 3u) * 4u + vown;
-                            const float2 v0 = lds64(va), v1 = lds64(va + vrow);
-                            s00 = fma2(A.c0 + v0.x, lo2(m0), s00);
-                            s01 = fma2(A.c0 + v0.y, hi2(m0), s01);
-                            s10 = fma2(A.c0 + v1.x, lo2(m1), s10);
-                            s11 = fma2(A.c0 + v1.y, hi2(m1), s11);
-                        }
                         const uint32_t T = st + (uint32_t)(R + ty) * rowb;
                         slabx_x(T, xc, A, m0, s00, s01);
                         slabx_x(T + rowb, xc, A, m1, s10, s11);
@@ -311,6 +305,14 @@ cheb_slabx_kernel(const float2* __restrict__ Y, const float2* __restrict__ Yprev
                             s01 = fma2v(A.cz[r], add2(hi2(u0), hi2(d0)), s01);
                             s10 = fma2v(A.cz[r], add2(lo2(u1), lo2(d1)), s10);
                             s11 = fma2v(A.cz[r], add2(hi2(u1), hi2(d1)), s11);
+                        }
+                        {   // the diagonal, by far the largest term, comes last: a sum is rounded to what it already holds
+                            const uint32_t va = st + A.off_v + ((g0 + A.vmis) & 3u) * 4u + vown;
+                            const float2 v0 = lds64(va), v1 = lds64(va + vrow);
+                            s00 = fma2(A.c0 + v0.x, lo2(m0), s00);
+                            s01 = fma2(A.c0 + v0.y, hi2(m0), s01);
+                            s10 = fma2(A.c0 + v1.x, lo2(m1), s10);
+                            s11 = fma2(A.c0 + v1.y, hi2(m1), s11);
                         }
                         float2 t00 = make_float2(0.f, 0.f), t01 = t00, t10 = t00, t11 = t00;
                         if (PREV) {
