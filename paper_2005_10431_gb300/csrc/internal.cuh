@@ -349,6 +349,8 @@ void launch_slab_variant(sdft_ctx* c, int kpt, const float2* Y, const float2* Yp
                          bool timed);
 // ---- stencil_slabx.cu: the same for any even n1 --------------------------------------------
 bool slabx_ok(const sdft_ctx* c, int ncolE);
+// no column, row or brick tile is faster: up to four KB slots, or one more than are staged, slabs of eight rows or more and no thin axis
+bool slabx_safe(const sdft_ctx* c, int ncolE);
 void launch_slabx(sdft_ctx* c, int kpt, const float2* Y, const float2* Yprev, float2* Ynext, int ncolE, const float* V,
                   const float2* kbC, double alpha, double beta, double shift, bool kin, bool timed);
 // sticky device flag (int) set by a stencil launch whose bounded mbarrier wait gave up

@@ -52,11 +52,15 @@ constexpr int kNReal = sizeof(kReal) / sizeof(kReal[0]);
 constexpr int kNCplx = sizeof(kCplx) / sizeof(kCplx[0]);
 }  // namespace
 
-// Real blocks with rows of 44 points and more (even): only the slab tiles are timed.  us a step, slab and best column, row
-// or brick tile: 80^3, 180 columns 294 and 668; 82 x 82 x 76, 176 columns 358 and 706; 96^3, 300 columns 915 and 1600;
-// 64 x 60 x 60, 66 columns 63 and 115; 48^3, 32 columns 23 and 27.  Shorter rows: 40^3 20.7 and 21.9, 36^3 19.0 and
-// 18.9, 20^3 27 and 18.
-static bool long_rows(const sdft_ctx* c, bool cplx, int ncolE) { return !cplx && c->n[0] >= 44 && slabx_ok(c, ncolE); }
+// Real blocks with rows of 44 points and more (even) for which slabx_safe() holds: only the slab tiles are timed.  us a
+// step, slab and best column, row or brick tile: 80^3, 180 columns 294 and 668; 82 x 82 x 76, 176 columns 358 and 706;
+// 96^3, 300 columns 915 and 1600; 64 x 60 x 60, 66 columns 63 and 115; 48^3, 32 columns 23 and 27; 160 x 40 x 40, 60
+// columns (4 slots) 119 and 132.  Shorter rows: 40^3 20.7 and 21.9, 36^3 19.0 and 18.9, 20^3 27 and 18.  Where it does not
+// hold: KB slots past the staged ones (four at most) are read from L2 by few threads, 64 x 60 x 60, 80 columns with 5, 9,
+// 21 slots 132 and 153, 221 and 175, 501 and 238; 80^3, 140 columns with 6, 52 slots 650 and 538, 4290 and 990; slabs of
+// 6, 4, 2 rows re-read their halo, 200 x 40 x 40 157 and 150, 256 x 40 x 40 218 and 205, 400 x 30 x 30 294 and 175; thin
+// axes do too, 60 x 7 x 400 160 and 121.
+static bool long_rows(const sdft_ctx* c, bool cplx, int ncolE) { return !cplx && c->n[0] >= 44 && slabx_safe(c, ncolE); }
 
 // Calls too small to be timed take a brick tile: 37 x 41 x 45 points, 20 columns: 15.4 us a step, 31 with the column
 // tile; 40^3, 28 columns: 20 and 26; 48^3, 40 columns: 35 and 66.  Bricks of 8 planes need two CTAs an SM, else 4.

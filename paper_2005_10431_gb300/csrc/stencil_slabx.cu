@@ -398,6 +398,14 @@ bool slabx_ok(const sdft_ctx* c, int ncolE) {
     return s.ty >= 2 && s.depth >= 3 && c->ng < (1LL << 31) && (long long)ncolE * c->n[2] < (1LL << 30);
 }
 
+bool slabx_safe(const sdft_ctx* c, int ncolE) {
+    if (!slabx_ok(c, ncolE)) return false;
+    int S = 0;
+    for (const KBTables& kb : c->kb) S = std::max(S, kb.S);
+    const SlabxShape s = slabx_shape(c, S);
+    return S <= std::max(4, s.nst + 1) && s.ty >= 8 && c->n[1] >= 2 * R && c->n[2] >= 2 * R;
+}
+
 void launch_slabx(sdft_ctx* c, int kpt, const float2* Y, const float2* Yprev, float2* Ynext, int ncolE, const float* V,
                   const float2* kbC, double alpha, double beta, double shift, bool kin, bool timed) {
     SDFT_REQUIRE(kin && V != nullptr, SDFT_ERR_INVALID_ARG, "slab stencil tile needs V and the kinetic term");
