@@ -947,7 +947,7 @@ struct StepVariant {
 
 // Stencil tile autotuner: time every compiled variant on the real operands (Ynext is rewritten by
 // the chosen variant afterwards) and keep the fastest for this context.  SDFT_STENCIL_VARIANT=k
-// forces variant k.  Small problems use variant 0 without timing.
+// forces variant k.  Small problems are not timed (-1).
 template <typename E>
 // proj (not null): the caller also needs the KB coefficients of the step's output, so each variant is
 // timed with them: followed by the separate projection pass `project` into proj, and, where the
@@ -963,7 +963,7 @@ int autotune_stencil(sdft_ctx* c, const StepVariant<E>* table, int nvar, int kpt
         const int v = atoi(env);
         if (v >= 0 && v < nvar && usable(v)) return v;
     }
-    if (nvar == 1 || (double)c->ng * ncolE < 4e6 || V == nullptr) return -1;   // not tuned: caller uses 0
+    if (nvar == 1 || (double)c->ng * ncolE < 4e6 || V == nullptr) return -1;   // not timed: the caller's rule decides
     cudaEvent_t a, b;
     SDFT_CUDA(cudaEventCreate(&a));
     SDFT_CUDA(cudaEventCreate(&b));
@@ -985,26 +985,43 @@ int autotune_stencil(sdft_ctx* c, const StepVariant<E>* table, int nvar, int kpt
         }
         return done;
     };
+    auto timed = [&](int v, bool fuse, int runs) {   // ms a step
+        SDFT_CUDA(cudaEventRecord(a, c->stream));
+        for (int q = 0; q < runs; ++q) run(v, fuse);
+        SDFT_CUDA(cudaEventRecord(b, c->stream));
+        SDFT_CUDA(cudaEventSynchronize(b));
+        float ms = 0.f;
+        SDFT_CUDA(cudaEventElapsedTime(&ms, a, b));
+        return ms / (float)runs;
+    };
+    // Every variant is run twice, the second time on the clock; only one within 15 % of the best so far, and that best
+    // itself, run twice more.  The last variants of a table come first: they are the faster ones, and most of the
+    // others then stop after their two runs.  First call of a context on odd rows, ms, when every variant ran four times
+    // and with the column tiles first: 65 x 63 x 61, 80 columns 13.9, 9.0 now; 81^3, 180 columns 63 and 38; the same
+    // 65 x 63 x 61 with Bloch phases 11.0 and 6.0.
     bool best_fused = false;
-    for (int v = 0; v < nvar; ++v) {
+    int best_runs = 0;
+    for (int v = nvar - 1; v >= 0; --v) {
         if (!(candidates >> v & 1) || !usable(v)) continue;
         for (int fuse = 0; fuse < (proj != nullptr ? 2 : 1); ++fuse) {
             const bool f = run(v, fuse != 0);   // warm-up
             if (fuse && !f) break;              // no fused projection in this variant
-            float ms = 0.f;
-            for (int r = 1; r <= 2; ++r) {      // one run, then two more unless it was far from the best
-                SDFT_CUDA(cudaEventRecord(a, c->stream));
-                for (int q = 0; q < r; ++q) run(v, fuse != 0);
-                SDFT_CUDA(cudaEventRecord(b, c->stream));
-                SDFT_CUDA(cudaEventSynchronize(b));
-                SDFT_CUDA(cudaEventElapsedTime(&ms, a, b));
-                ms /= (float)r;
-                if (ms > 1.25f * best_ms) break;
+            float ms = timed(v, fuse != 0, 1);
+            int runs = 1;
+            if (ms > 1.15f * best_ms) continue;
+            if (ms > 0.87f * best_ms) {
+                ms = timed(v, fuse != 0, 2);
+                runs = 2;
+                if (best_runs == 1) {
+                    best_ms = timed(best, best_fused, 2);
+                    best_runs = 2;
+                }
             }
             if (ms < best_ms) {
                 best_ms = ms;
                 best = v;
                 best_fused = fuse != 0;
+                best_runs = runs;
             }
         }
     }
