@@ -64,6 +64,7 @@ struct KBTables {
     double* val64 = nullptr;  // [natom*cap] real chi (double)  or [2*natom*cap] complex beta
     float* val32 = nullptr;   // same in float
     int S = 0;                // slots per grid point
+    double mean = 0.0;        // slots used at a point on average: the spheres' volume over the cell's
     int* pcnt = nullptr;      // [ng]
     int* patom = nullptr;     // [S*ng] atom of slot s at point g, -1 if unused (sorted by atom)
     double* pval64 = nullptr; // [S*ng] (x2 complex)

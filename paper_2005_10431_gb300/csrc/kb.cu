@@ -239,6 +239,8 @@ void build_kb_tables(sdft_ctx* c, int kpt) {
         cap = std::max(cap, B.dim[0] * B.dim[1] * B.dim[2]);
     }
     T.cap = std::max(cap, 1);
+    T.mean = 0.0;
+    for (const AtomBox& B : boxes) T.mean += 4.0 / 3.0 * M_PI * B.rc * B.rc * B.rc / (c->L[0] * c->L[1] * c->L[2]);
     const size_t ent = (size_t)c->natom * T.cap;
     const int vw = T.cplx ? 2 : 1;
     T.cnt = (int*)ctx_alloc(c, sizeof(int) * std::max(1, c->natom));

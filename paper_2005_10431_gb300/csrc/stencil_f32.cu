@@ -62,13 +62,24 @@ constexpr int kNCplx = sizeof(kCplx) / sizeof(kCplx[0]);
 // axes do too, 60 x 7 x 400 160 and 121.
 static bool long_rows(const sdft_ctx* c, bool cplx, int ncolE) { return !cplx && c->n[0] >= 44 && slabx_safe(c, ncolE); }
 
+// Cells whose projectors overlap so much that the column tile is ahead of the bricks, which read the KB slots with few
+// warps: more than seven slots at a point on average, and a block that fills the GPU with column tiles.  us a step, column
+// tile and brick of 8 planes at 6, 8, 12 slots: 40^3, 20 columns 51 and 45, 59 and 62, 57 and 81; 10 columns 45 and 27, 53
+// and 37, 50 and 47; Bloch, 60 x 50 x 50, 20 columns 155 and 157, 190 and 196, 243 and 291; 40^3, 20 columns 108 and
+// 74, 121 and 100, 130 and 129.
+static bool dense_kb(const sdft_ctx* c, bool cplx, int ncolE) {
+    double mean = 0.0;
+    for (const KBTables& kb : c->kb) mean = std::max(mean, kb.mean);
+    return mean > 7.0 && (double)c->ng * ncolE > (cplx ? 2.5e6 : 5e5);
+}
+
 // Calls too small to be timed take a brick tile: 37 x 41 x 45 points, 20 columns: 15.4 us a step, 31 with the column
 // tile; 40^3, 28 columns: 20 and 26; 48^3, 40 columns: 35 and 66.  Bricks of 8 planes need two CTAs an SM, else 4.
 // (The slab would take 29 us for the last of these, but the multi-cell filter runs bricks, and a cell gets the same bits
 // from it as from its own filter.)
 static int small_variant(const sdft_ctx* c, bool cplx, int ncolE) {
     const int v8 = cplx ? kCplxBrick8 : kRealBrick8;
-    if (!brick_ok<float2, 8>(c, ncolE)) return 0;
+    if (!brick_ok<float2, 8>(c, ncolE) || dense_kb(c, cplx, ncolE)) return 0;
     const BrickTile t = brick_tile(c->n[0], c->n[1]);
     const long long ctas8 = (long long)t.tiles_x * t.tiles_y * ((c->n[2] + 7) / 8) * ncolE;
     return ctas8 >= 2 * 152 ? v8 : v8 + 1;
@@ -230,10 +241,12 @@ void chebyshev_filter_multi(const std::vector<sdft_ctx*>& ctxs, const std::vecto
     SDFT_REQUIRE(n >= 1 && n <= MULTI_MAX, SDFT_ERR_INVALID_ARG, "multi-cell launch takes 1..64 cells");
     for (int i = 0; i < n; ++i)
         SDFT_REQUIRE(b[i] > a[i] && a[i] > a0[i], SDFT_ERR_INVALID_ARG, "filter bounds must satisfy a0 < a < b");
-    // cells whose KB coefficients do not fit beside a brick (some 5000 atoms and more) are filtered on their own
+    // cells whose KB coefficients do not fit beside a brick (some 5000 atoms and more), or that fill the GPU and take
+    // another tile (dense_kb), are filtered on their own
     std::vector<int> fit;
     for (int i = 0; i < n; ++i)
-        if (brick_ok<float2, MULTI_ZC>(ctxs[i], ctxs[i]->nfilt / 2)) fit.push_back(i);
+        if (brick_ok<float2, MULTI_ZC>(ctxs[i], ctxs[i]->nfilt / 2) && !dense_kb(ctxs[i], false, ctxs[i]->nfilt / 2))
+            fit.push_back(i);
     if ((int)fit.size() < n) {
         std::vector<sdft_ctx*> cs;
         std::vector<const void*> xs;

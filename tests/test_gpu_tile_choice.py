@@ -20,10 +20,10 @@ def sd():
     return m
 
 
-def _filter(sd, n, natom, spread, ns, calls=1, kred=None):
+def _filter(sd, n, natom, spread, ns, calls=1, kred=None, Z=4.0):
     """tile of a filter of `ns` columns, and the launches of each of `calls` calls"""
     cell = workloads.small_cell(npts=8, L=4.0, natom=natom, seed=3, nstates=ns)
-    cell.n, cell.L = n, tuple(0.2565 * k for k in n)
+    cell.n, cell.L, cell.species = n, tuple(0.2565 * k for k in n), [workloads.Species(Z=Z)]
     cell.pos = np.random.default_rng(natom).uniform(0, spread, (natom, 3)) * np.array(cell.L)
     ctx = sd.sdft_create(cell.L, cell.n, cell.pos, cell.types, cell.species,
                          dict(nstates=ns, precision=sd.SDFT_MIXED, mix_hist=1), kpts=kred)
@@ -48,6 +48,15 @@ def _filter(sd, n, natom, spread, ns, calls=1, kred=None):
 def test_slab_tiles_where_they_are_ahead(sd, n, natom, spread, ns, slab):
     name, _ = _filter(sd, n, natom, spread, ns)
     assert name.startswith("slab") == slab, name
+
+
+@pytest.mark.parametrize("n,natom,tile", [
+    ((40, 40, 40), 8, "brick"), ((40, 40, 40), 110, "col"),   # 0.8 and 11 slots at a point on average
+    ((24, 24, 24), 24, "brick")])                             # 12, but too small a block to fill the GPU
+def test_untimed_calls(sd, n, natom, tile):
+    name, launches = _filter(sd, n, natom, 1.0, 20, calls=2, Z=1.8 * 20 / natom if natom > 8 else 4.0)
+    assert name.startswith(tile)
+    assert launches[0] == launches[1]
 
 
 # seven column tiles (Bloch blocks: two) run four times each, with a projection (Bloch: none) after every run, were 56 and 8
