@@ -154,9 +154,14 @@ def measured_peaks():
     return 6800.0, "fallback"
 
 
+# sources of the slab tiles whose DRAM traffic is on record
+STENCIL_SOURCES = ("stencil_impl.cuh", "stencil_brick.cuh", "stencil_f32.cu", "stencil_tma.cu", "stencil_ptx.cuh",
+                   "stencil_slabx.cu")
+
+
 def stencil_source_hash():
     h = hashlib.sha256()
-    for f in ("stencil_impl.cuh", "stencil_f32.cu", "stencil_tma.cu"):
+    for f in STENCIL_SOURCES:
         h.update(open(os.path.join(ROOT, "paper_2005_10431_gb300", "csrc", f), "rb").read())
     return h.hexdigest()[:16]
 
