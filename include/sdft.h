@@ -202,7 +202,7 @@ sdft_status sdft_scf(sdft_ctx* ctx, sdft_result* out);
  * running context computes its potential, then the CheFSI passes: cells in mixed precision with
  * one real Gamma-point problem, sharing one stream, with equal degree and pass count are filtered
  * together (sdft_chebyshev_filter_multi: one KB projection and one stencil launch per Chebyshev
- * step for all of them, column-tile stencil), each followed by its own Rayleigh-Ritz; other
+ * step for all of them, brick-tile stencil), each followed by its own Rayleigh-Ritz; other
  * contexts run their passes alone.  A context stops at its own convergence or max_scf.
  * out: host array of n results, filled for every context.  Returns the first non-OK status in
  * context order (NOT_CONVERGED if a context did not converge); an error inside any context

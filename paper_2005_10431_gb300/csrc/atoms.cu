@@ -268,7 +268,7 @@ overlap_energy_kernel(const PairAtom* __restrict__ at, int natom, int m1, int m2
         const double v[3] = {A.pos[0] - B.pos[0] - t0 * L1, A.pos[1] - B.pos[1] - t1 * L2, A.pos[2] - B.pos[2] - t2 * L3};
         const double d2 = v[0] * v[0] + v[1] * v[1] + v[2] * v[2];
         if (d2 > rmax * rmax) continue;
-        // erfc(q) and exp(-q^2) are below 1e-44 past q = 10: no bit of a sum of larger terms, and such terms alone are
+        // erfc(q) and exp(-q^2) are below 4e-44 past q = 10: no bit of a sum of larger terms, and such terms alone are
         // no energy
         const double s2 = 2.0 * (A.r_loc * A.r_loc + B.r_loc * B.r_loc);
         if (d2 > 100.0 * s2) continue;

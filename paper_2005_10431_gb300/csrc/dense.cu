@@ -172,8 +172,8 @@ gram_kernel(const void* __restrict__ Y, const void* __restrict__ HY, int ncol, l
 // Sum the split-K partials (upper triangle) and mirror to a full Hermitian matrix.  A 20-state matrix has 210
 // sums of up to 432 terms: one thread per element walking through them was one memory latency per term (310 us
 // complex, 77 us for 8 states).  LANES threads now share an element's terms of one matrix, eight loads in flight
-// each: 20 complex columns 310 -> 14 us, 8 FP64 columns 77 -> 28 us.  FP64 kinds keep one thread per sum (LANES = 1, 16 loads in flight) and with it the order of
-// the additions, so FP64 results are the same bit for bit as before; the FP32 kinds' partials carry FP32 rounding.
+// each: 20 complex columns 310 -> 14 us, 8 FP64 columns 77 -> 28 us.  FP64 kinds keep one thread per sum (LANES = 1, 16 loads
+// in flight) and with it the order of the additions; the FP32 kinds' partials carry FP32 rounding.
 // grid.y: matrix (M, Hs); W = 2 for complex.
 template <int LANES, int W>
 __global__ void __launch_bounds__(256)

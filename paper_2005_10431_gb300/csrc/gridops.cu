@@ -1,5 +1,5 @@
-// Grid-level FP64 kernels of the SCF (paper Sec. 2.1): Perdew-Zunger LDA, the AAR Poisson solver, density from orbitals (Eq. 2), Fermi-Dirac
-// occupations, Pulay mixing, reductions and Hellmann-Feynman forces.
+// Grid-level FP64 kernels of the SCF (paper Sec. 2.1): Perdew-Zunger LDA, the AAR Poisson solver, density from
+// orbitals (Eq. 2), Fermi-Dirac occupations, Pulay mixing, reductions and Hellmann-Feynman forces.
 #include "internal.cuh"
 
 #include <algorithm>

@@ -7,8 +7,8 @@
 // M applies one V-cycle of the second-order (7-point) Laplacian A2 on a hierarchy of grids that
 // halves every dimension while it is even: red-black Gauss-Seidel smoothing, full-weighting
 // restriction of the residual, trilinear prolongation, and on the coarsest grid (at most 512
-// points, or up to 16 384 when a dimension turns odd earlier) a fixed number of Chebyshev iterations for the known spectrum of A2 run by one CTA out
-// of shared memory.  A2 and A share their low-frequency spectrum; at the highest grid frequency the
+// points, or up to 16 384 when a dimension turns odd earlier) a fixed number of Chebyshev
+// iterations for the known spectrum of A2, run by one CTA out of shared memory.  A2 and A share their low-frequency spectrum; at the highest grid frequency the
 // order-12 symbol is about 2.5 times the second-order one, so the preconditioned operator M A
 // keeps its eigenvalues in a small interval and AAR reaches a 1e-3 reduction in a few iterations
 // instead of the hundreds the Jacobi scaling needs (its iteration count grows with the grid).

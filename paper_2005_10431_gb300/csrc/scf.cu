@@ -893,7 +893,7 @@ sdft_status run_scf(sdft_ctx* c, sdft_result* out) {
 // together -- one grouped KB projection and one stencil launch per Chebyshev step for all of
 // them -- followed by each cell's Rayleigh-Ritz; then every context's density, energy and mixing.
 // A context leaves the lockstep when it converges or reaches its max_scf.  The results are
-// those of running each context alone with the column-tile stencil.
+// those of running each context alone with a brick or column tile (the same sums in the same order).
 sdft_status run_batch_scf(const std::vector<sdft_ctx*>& ctxs, sdft_result* out) {
     const int n = (int)ctxs.size();
     std::vector<std::unique_ptr<ScfRun>> runs;
