@@ -16,7 +16,7 @@
 // rows reads 32 consecutive columns' banks without conflicts.
 // Sums are formed in the column tile's order: real blocks get the same bits.  (Bloch blocks round the product of two
 // phase factors differently at the cell's edges: 1e-16 of the largest value in FP64, 6e-8 in FP32.)
-// Measured, column tile -> brick, us per step: 24^3, FP64, 8 columns 87 -> 12; 37 x 41 x 45, FP32, 20 columns 31 -> 15;
+// Measured, column tile -> brick, us per step (kernel time): 24^3, FP64, 8 columns 87 -> 12; 37 x 41 x 45, FP32, 20 columns 31 -> 15;
 // 40^3, Bloch, 20 columns 59 -> 25; 48^3, 40 columns 66 -> 35; 32 cells of 24 to 48 points in one launch 427 -> 310.
 // Bound by issue and shared-memory reads of one tile at a time (two CTAs per SM).  Staging V_eff and the KB slots in
 // shared memory as well was slower (15 -> 20, 25 -> 36, 310 -> 385).

@@ -64,7 +64,8 @@ void launch_cheb_step<double>(sdft_ctx* c, int kpt, const double* Y, const doubl
         count_launch(c);
         return;
     }
-    // The brick at every size it takes, us per step (column tile -> brick): 24^3 x 8 90 -> 16, 36^3 x 24 220 -> 125,
+    // The brick at every size it takes, us per step between events, some 4 us more than
+    // the kernel (column tile -> brick): 24^3 x 8 90 -> 16, 36^3 x 24 220 -> 125,
     // 64^3 x 64 1487 -> 1439, 80^3 x 140 7389 -> 6081
     if (brick_ok<double, 4>(c, ncolE) && V != nullptr) {
         launch_brick<double, false, 4, 2>(c, kpt, Y, Yprev, Ynext, ncolE, V, kbC, alpha, beta, shift, with_kinetic, true);

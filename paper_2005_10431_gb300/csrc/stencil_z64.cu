@@ -8,7 +8,7 @@ template <>
 void launch_cheb_step<double2>(sdft_ctx* c, int kpt, const double2* Y, const double2* Yprev, double2* Ynext, int ncolE,
                                const double* V, const double2* kbC, double alpha, double beta, double shift,
                                bool with_kinetic) {
-    // us per step (column tile -> brick): 24^3 x 8 210 -> 33, 36^3 x 24 570 -> 255, 48^3 x 24 833 -> 550
+    // us per step between events (column tile -> brick): 24^3 x 8 210 -> 33, 36^3 x 24 570 -> 255, 48^3 x 24 833 -> 550
     if (brick_ok<double2, 4>(c, ncolE) && V != nullptr) {
         launch_brick<double2, true, 4, 2>(c, kpt, Y, Yprev, Ynext, ncolE, V, kbC, alpha, beta, shift, with_kinetic, true);
         return;
