@@ -6,7 +6,7 @@
 //   2. Cholesky M' = L L^H
 //   3. A = L^-1 H' L^-H (two triangular solves, then symmetrised)
 //   4. cyclic Jacobi on A with the round-robin (tournament) order: n/2 disjoint rotations per
-//      round, applied to 2 x 2 blocks from both sides; sweeps until no rotation is needed
+//      round, applied from both sides; sweeps until no rotation is needed
 //   5. eigenvalues ascending, Q = D L^-H V
 // Q overwrites Hs (column-major, eigenvector j in column j), eig ascending; info[p] = 0, or k+1
 // if the equilibrated M is not positive definite at column k.
@@ -74,9 +74,12 @@ __device__ __forceinline__ int rr_pos(int i, int r, int m) { return i == 0 ? 0 :
 
 // Bound by the chains of dependent FP64 operations of one small problem (a division or square root is some 400 cycles,
 // a product or sum 45), so: real problems take no imaginary parts and no modulus or phase (half of a rotation's square
-// roots and divisions), the diagonal of L is inverted once, and a thread applies both sides of a round's rotations to its
-// 2 x 2 block of A, with one barrier where the column and the row pass had two.  The same operations in the same order:
-// no bit of the result depends on it.  n = 8, one real problem: 201 -> 129 us.
+// roots and divisions) and apply both sides of a round's rotations to 2 x 2 blocks of A, a thread each, with one barrier
+// where the column and the row pass have two; complex problems keep the two passes, because sixteen complex products
+// in a block's chain take longer than the passes' twelve (n = 8, 20, 33: 277, 1192, 3975 us in blocks, 265, 1117, 3849 in
+// passes).  The diagonal of L is inverted once.  The same operations in the same order: real and complex results are
+// the same bit for bit as those of one kernel in complex arithmetic.  Real, n = 8, 33, 64: 277, 4110, 20529 -> 191, 2067,
+// 8700 us a call.
 template <typename T>
 __global__ void __launch_bounds__(256)
 batched_geig_kernel(double* const* __restrict__ Ms, double* const* __restrict__ Hss, double* const* __restrict__ eigs,
@@ -206,54 +209,86 @@ batched_geig_kernel(double* const* __restrict__ Ms, double* const* __restrict__ 
                 }
             }
             __syncthreads();
-            // A <- U^H A U by 2 x 2 blocks (rows of pair i, columns of pair k), V <- V U
-            for (int e = tid; e < npair * npair; e += NT) {
-                const int k = e / npair, i = e - k * npair;
-                const int a = rp[k], b = rq[k], u = rp[i], v = rq[i];
-                const bool bc = b < n, bv = v < n;     // odd n: one pair has a single member
-                const bool rotc = bc && rs[k] != 0.0, rotr = bv && rs[i] != 0.0;
-                if (!rotc && !rotr) continue;
-                T ua = AT(A, u, a), ub = elem<T>(0.0), va = ub, vb = ub;
-                if (bc) ub = AT(A, u, b);
-                if (bv) va = AT(A, v, a);
-                if (bc && bv) vb = AT(A, v, b);
-                if (rotc) {
+            if constexpr (sizeof(T) == sizeof(Cx)) {
+                // columns: A <- A U, V <- V U
+                for (int e = tid; e < npair * n; e += NT) {
+                    const int k = e / n, row = e - k * n;
+                    if (rq[k] >= n || rs[k] == 0.0) continue;
+                    const int a = rp[k], b = rq[k];
                     const double c = rc[k], s = rs[k];
                     const T ce = conj(re[k]);
                     const T upp = elem<T>(c), upq = elem<T>(s), uqp = (-s) * ce, uqq = c * ce;
-                    const T x = ua * upp + ub * uqp, y = ua * upq + ub * uqq;
-                    ua = x;
-                    ub = y;
-                    const T z = va * upp + vb * uqp, w = va * upq + vb * uqq;
-                    va = z;
-                    vb = w;
+                    T x = AT(A, row, a), y = AT(A, row, b);
+                    AT(A, row, a) = x * upp + y * uqp;
+                    AT(A, row, b) = x * upq + y * uqq;
+                    x = AT(V, row, a);
+                    y = AT(V, row, b);
+                    AT(V, row, a) = x * upp + y * uqp;
+                    AT(V, row, b) = x * upq + y * uqq;
                 }
-                if (rotr) {
-                    const double c = rc[i], s = rs[i];
-                    const T ce = conj(re[i]);
+                __syncthreads();
+                // rows: A <- U^H A
+                for (int e = tid; e < npair * n; e += NT) {
+                    const int k = e / n, col = e - k * n;
+                    if (rq[k] >= n || rs[k] == 0.0) continue;
+                    const int a = rp[k], b = rq[k];
+                    const double c = rc[k], s = rs[k];
+                    const T ce = conj(re[k]);
                     const T upp = elem<T>(c), upq = elem<T>(s), uqp = (-s) * ce, uqq = c * ce;
-                    const T x = conj(upp) * ua + conj(uqp) * va, y = conj(upq) * ua + conj(uqq) * va;
-                    ua = x;
-                    va = y;
-                    const T z = conj(upp) * ub + conj(uqp) * vb, w = conj(upq) * ub + conj(uqq) * vb;
-                    ub = z;
-                    vb = w;
+                    const T x = AT(A, a, col), y = AT(A, b, col);
+                    AT(A, a, col) = conj(upp) * x + conj(uqp) * y;
+                    AT(A, b, col) = conj(upq) * x + conj(uqq) * y;
                 }
-                AT(A, u, a) = ua;
-                if (bc) AT(A, u, b) = ub;
-                if (bv) AT(A, v, a) = va;
-                if (bc && bv) AT(A, v, b) = vb;
-            }
-            for (int e = NT - 1 - tid; e < npair * n; e += NT) {   // from the other end: threads without a block first
-                const int k = e / n, row = e - k * n;
-                if (rq[k] >= n || (rs[k] == 0.0)) continue;
-                const int a = rp[k], b = rq[k];
-                const double c = rc[k], s = rs[k];
-                const T ce = conj(re[k]);
-                const T upp = elem<T>(c), upq = elem<T>(s), uqp = (-s) * ce, uqq = c * ce;
-                const T x = AT(V, row, a), y = AT(V, row, b);
-                AT(V, row, a) = x * upp + y * uqp;
-                AT(V, row, b) = x * upq + y * uqq;
+            } else {
+                // A <- U^H A U by 2 x 2 blocks (rows of pair i, columns of pair k), V <- V U
+                for (int e = tid; e < npair * npair; e += NT) {
+                    const int k = e / npair, i = e - k * npair;
+                    const int a = rp[k], b = rq[k], u = rp[i], v = rq[i];
+                    const bool bc = b < n, bv = v < n;     // odd n: one pair has a single member
+                    const bool rotc = bc && rs[k] != 0.0, rotr = bv && rs[i] != 0.0;
+                    if (!rotc && !rotr) continue;
+                    T ua = AT(A, u, a), ub = elem<T>(0.0), va = ub, vb = ub;
+                    if (bc) ub = AT(A, u, b);
+                    if (bv) va = AT(A, v, a);
+                    if (bc && bv) vb = AT(A, v, b);
+                    if (rotc) {
+                        const double c = rc[k], s = rs[k];
+                        const T ce = conj(re[k]);
+                        const T upp = elem<T>(c), upq = elem<T>(s), uqp = (-s) * ce, uqq = c * ce;
+                        const T x = ua * upp + ub * uqp, y = ua * upq + ub * uqq;
+                        ua = x;
+                        ub = y;
+                        const T z = va * upp + vb * uqp, w = va * upq + vb * uqq;
+                        va = z;
+                        vb = w;
+                    }
+                    if (rotr) {
+                        const double c = rc[i], s = rs[i];
+                        const T ce = conj(re[i]);
+                        const T upp = elem<T>(c), upq = elem<T>(s), uqp = (-s) * ce, uqq = c * ce;
+                        const T x = conj(upp) * ua + conj(uqp) * va, y = conj(upq) * ua + conj(uqq) * va;
+                        ua = x;
+                        va = y;
+                        const T z = conj(upp) * ub + conj(uqp) * vb, w = conj(upq) * ub + conj(uqq) * vb;
+                        ub = z;
+                        vb = w;
+                    }
+                    AT(A, u, a) = ua;
+                    if (bc) AT(A, u, b) = ub;
+                    if (bv) AT(A, v, a) = va;
+                    if (bc && bv) AT(A, v, b) = vb;
+                }
+                for (int e = NT - 1 - tid; e < npair * n; e += NT) {   // from the other end: threads without a block first
+                    const int k = e / n, row = e - k * n;
+                    if (rq[k] >= n || (rs[k] == 0.0)) continue;
+                    const int a = rp[k], b = rq[k];
+                    const double c = rc[k], s = rs[k];
+                    const T ce = conj(re[k]);
+                    const T upp = elem<T>(c), upq = elem<T>(s), uqp = (-s) * ce, uqq = c * ce;
+                    const T x = AT(V, row, a), y = AT(V, row, b);
+                    AT(V, row, a) = x * upp + y * uqp;
+                    AT(V, row, b) = x * upq + y * uqq;
+                }
             }
             __syncthreads();
         }
